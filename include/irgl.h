@@ -54,7 +54,8 @@ typedef enum {
   IRGL_BFS = 0,  /* level assignment, Sec. 4.1 level-by-level BFS listing */
   IRGL_SSSP = 1, /* data-driven edge relaxation with atomicMin */
   IRGL_CC = 2,   /* min-label propagation over a symmetric graph */
-  IRGL_CC_JUMP = 3 /* same labels by min-hooking and pointer jumping (persistent Iterate only) */
+  IRGL_CC_JUMP = 3 /* same labels by hooking roots and pointer jumping (persistent Iterate only; CTAs of
+                      1024 whatever the tuning says, two rounds: link every edge, then flatten) */
 } irgl_kernel;
 
 /* How Iterate drives the kernel (Sec. 4.4 kernel invocations). */

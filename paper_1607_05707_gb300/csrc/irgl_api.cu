@@ -821,6 +821,7 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   s = ensure_workspace(ctx, g->n, k != IRGL_BFS, far, vis, packed, use_local ? sub_rounds + 1u : 1u);
   if (s != IRGL_OK) return s;
   const uint32_t op = (use_local && k == IRGL_BFS) ? OP_BFSR : op_of(k);
+  if (k == IRGL_CC_JUMP) t.cta_size = kUfCta;  // its vertex blocks fill an SM's shared memory: one CTA each
   if (k == IRGL_CC_JUMP && mode != IRGL_PERSISTENT)
     return fail(IRGL_ERR_UNSUPPORTED, "pointer-jumping CC runs only as a persistent Iterate");
   KParams p = make_params(ctx, g, state_dev, t);

@@ -678,7 +678,7 @@ struct RoundCtx {
   Out far_out;
   uint32_t* far_stamp;
   uint32_t phase;                 // far-list dedup id of the current phase
-  uint32_t* changes;              // pointer-jumping CC: hooks that lowered a parent (shared memory)
+  uint32_t* changes;              // pointer-jumping CC: roots hooked (shared memory)
   unsigned long long* mf;         // direction-optimising BFS: out-degrees of pushed vertices (shared memory)
   const uint32_t* row_ptr;        //   and the row offsets to take them from
   uint32_t* vis;                  // BFS visited bitmap, or nullptr
@@ -731,6 +731,57 @@ __device__ __forceinline__ uint32_t load_cur(const RoundCtx& rc, const uint32_t*
   return __ldcg(state + v);
 }
 
+// Union-find over parent[] (parent[x] <= x, roots point at themselves), in
+// global or (SH) shared memory. Parents only ever move to smaller ancestors, so
+// every loop below ends. Global reads go through L1: a stale parent is still an
+// ancestor, and the CAS that hooks a root decides on the current value; read from
+// L2, the few roots of a large component are one line that every warp of the grid
+// queues for. uf_climb: the root above x, whose parent was read as `f`, halving
+// the path on the way (only non-roots are written, and only with their ancestors,
+// so a lost store just leaves a longer path).
+template <bool SH>
+__device__ __forceinline__ uint32_t uf_ld(const uint32_t* p) {
+  return SH ? *reinterpret_cast<const volatile uint32_t*>(p) : __ldca(p);
+}
+template <bool SH>
+__device__ __forceinline__ uint32_t uf_climb(uint32_t* parent, uint32_t x, uint32_t f) {
+  uint32_t prev = x;
+  while (f != prev) {
+    const uint32_t up = uf_ld<SH>(parent + f);
+    if (up == f) return f;
+    if (SH) *reinterpret_cast<volatile uint32_t*>(parent + prev) = up;
+    else __stcg(parent + prev, up);
+    prev = f;
+    f = up;
+  }
+  return f;
+}
+
+// Join the trees of a and of rb, a (possibly former) root: the larger root is
+// hooked under the smaller one by a CAS that succeeds only on a root; a failed CAS
+// tells the parent it got meanwhile, and the climb from there reads L2.
+// Returns the joined tree's smaller end, an ancestor of a.
+template <bool SH>
+__device__ __forceinline__ uint32_t uf_link(uint32_t* parent, uint32_t a, uint32_t rb, uint32_t& hooked) {
+  uint32_t ra = uf_climb<SH>(parent, a, uf_ld<SH>(parent + a));
+  while (ra != rb) {
+    const uint32_t hi = max(ra, rb), lo = min(ra, rb);
+    uint32_t old = atomicCAS(parent + hi, hi, lo);
+    if (old == hi) {
+      ++hooked;
+      return lo;
+    }
+    for (;;) {
+      const uint32_t up = SH ? uf_ld<SH>(parent + old) : __ldcg(parent + old);
+      if (up == old) break;
+      old = up;
+    }
+    ra = old;
+    rb = lo;
+  }
+  return ra;
+}
+
 // decide() with the near-far routing (SSSP, CC): 0 = no push, 1 = push to this
 // round's out-worklist, 2 = push to the far list. Near pushes dedup on the
 // round stamp, far pushes on the phase stamp, so a vertex improved first above
@@ -740,10 +791,10 @@ __device__ __forceinline__ uint32_t decide_route(uint32_t op_rt, uint32_t* state
                                                  uint32_t val, int32_t wt, uint32_t cur, const RoundCtx& rc,
                                                  uint32_t sb, uint32_t& nd_out) {
   if (OP == OP_CCJ) {
-    // hook: the larger of the two endpoints' parents is pointed at the smaller one
-    if (val == cur) return 0u;
-    const uint32_t lo = min(val, cur), hi = max(val, cur);
-    if (atomicMin(state + hi, lo) > lo) atomicAdd(rc.changes, 1u);
+    // link the roots of u (= val) and v; each edge is taken from its larger end
+    uint32_t hooked = 0;
+    if (v < val) uf_link<false>(state, val, uf_climb<false>(state, v, cur), hooked);
+    if (hooked) atomicAdd(rc.changes, 1u);
     return 0u;
   }
   if (OP == OP_BFS) {
@@ -2495,86 +2546,235 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   persistent_exit<CTA>(sm, st, ok, rounds, last_out, ep0, esum, nullptr, 0);
 }
 
-// Connected components by min-hooking and pointer jumping, in one cooperative
-// launch. parent = state, initially parent[v] = v. Each iteration: (1) hook:
-// for every edge (u, v) with parents a = parent[u], b = parent[v], a != b,
-// atomicMin(parent[max(a,b)], min(a,b)); (2) shortcut: every vertex follows
-// its parent pointers to the root and stores it. Parents only decrease and
-// always name a vertex of the same component, so the first hook phase that
-// lowers nothing leaves every component pointing at one root, its minimum id:
-// the labels of min-label propagation in O(log n) iterations instead of
-// O(diameter) rounds.
-template <int CTA>
-__device__ __forceinline__ void cc_jump_persistent(const KParams& p, Smem<CTA>& sm) {
+// Connected components by hooking and pointer jumping, in one cooperative
+// launch. parent = state; parent[v] <= v always, a root is parent[v] == v, and
+// every link puts the larger of two roots under the smaller one (uf_link), so the
+// root of a tree is its smallest id. Every edge is taken from its larger end (a
+// symmetric graph holds both directions). Round 1: (a) each CTA takes blocks of
+// consecutive vertices, links the edges that stay inside a block in shared memory
+// and writes every vertex's parent, its block root; (b) after a barrier the edges
+// that leave a block downwards are linked in global memory. Round 2: every vertex
+// follows its parents to the root and stores it (skipped when nothing was hooked).
+//
+// What bounds it: the adjacency is streamed twice; the rest is chains of dependent
+// parent reads, and they are what costs: with every link in global memory a
+// 4096^2 mesh (a tenth of its edges missing) took 2.9 ms, 25 us per warp step, the
+// rows of a wave climbing through each other; one parent per hook and iteration
+// (the former kernel: four iterations of 0.42-1.23 ms) 2.83 ms; with blocks of
+// nine rows in shared memory (a climb step is 30 cycles, and one edge in eighteen
+// leaves its block) 0.44 ms: 0.23 for (a), 0.18 for (b), 0.03 for round 2.
+// Lists of at most kUfLane edges are walked by the lane that holds the vertex,
+// four columns in flight (no search for an edge's owner: mesh lists have two to
+// four entries); longer ones by the warp; those of kUfSplit edges or more by the
+// whole grid (big list), block edges included.
+constexpr uint32_t kUfLane = 16;
+constexpr uint32_t kUfSplit = 512;
+constexpr int kUfCta = 1024;
+constexpr uint32_t kUfTile = 40 * 1024;  // vertices of a block: 160 KB of shared memory beside the CTA's Smem
+
+// Vertices per block: the smallest number of blocks that is a multiple of the
+// grid and fits the tile (no CTA is left with one block more than the others),
+// but at least 1024, so that a small graph keeps some of its edges inside blocks.
+__device__ __forceinline__ uint32_t uf_block_size(uint32_t n, uint32_t grid) {
+  const unsigned long long tiles = static_cast<unsigned long long>(kUfTile) * grid;
+  const unsigned long long nb = max((n + tiles - 1u) / tiles, 1ull) * grid;
+  return min(max(static_cast<uint32_t>((n + nb - 1u) / nb), 1024u), kUfTile);
+}
+
+// Link the edges (u, v) of the vertices [lo, hi): inside the block (SH: v >= lo,
+// parents tile[] indexed from lo) or below it (v < lo, parents in p.state).
+template <bool SH>
+__device__ __forceinline__ void uf_edges(const KParams& p, Smem<kUfCta>& sm, const RoundCtx& rc, uint32_t lo, uint32_t hi,
+                                         uint32_t split, uint32_t* tile, uint32_t& edges, uint32_t& hooked) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t* const par = SH ? tile : p.state;
+  const uint32_t off = SH ? lo : 0u;
+  uint32_t nbeg = threadIdx.x < hi - lo ? __ldg(p.row_ptr + lo + threadIdx.x) : 0u;
+  uint32_t nend = threadIdx.x < hi - lo ? __ldg(p.row_ptr + lo + threadIdx.x + 1) : 0u;
+  for (uint32_t base = threadIdx.x & ~31u; base < hi - lo; base += kUfCta) {
+    const uint32_t u = lo + base + lane;
+    const uint32_t beg = nbeg, end = nend;
+    const bool more = base + kUfCta + lane < hi - lo;  // the next step's offsets, loaded a step ahead
+    nbeg = more ? __ldg(p.row_ptr + u + kUfCta) : 0u;
+    nend = more ? __ldg(p.row_ptr + u + kUfCta + 1) : 0u;
+    const uint32_t deg = end - beg;
+    if (!SH) edges += deg;
+    bool wide = deg > kUfLane;
+    if (!wide) {
+      uint32_t ru = u - off;
+      for (uint32_t e = beg; e < end; e += 4) {
+        uint32_t c[4], f[4];
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+          c[k] = e + k < end ? __ldg(p.col + e + k) : kInf;
+          if (SH ? (c[k] < lo || c[k] >= u) : c[k] >= lo) c[k] = kInf;
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) f[k] = c[k] != kInf ? uf_ld<SH>(par + (c[k] - off)) : 0u;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k)
+          if (c[k] != kInf) ru = uf_link<SH>(par, ru, uf_climb<SH>(par, c[k] - off, f[k]), hooked);
+      }
+    }
+    // lists for the whole grid: listed once (in the global pass), with every edge they have
+    bool big = rc.big.cap != 0 && deg >= split;
+    if (__any_sync(kFull, big)) {
+      if (SH) {
+        wide = wide && !big;
+      } else {
+        const unsigned long long mine = big ? ((1ull << 40) | deg) : 0ull;
+        const unsigned long long incl = warp_incl_scan64(mine);
+        const unsigned long long total = __shfl_sync(kFull, incl, 31);
+        unsigned long long at = 0;
+        if (lane == 31) {
+          at = atomicAdd(rc.big_ctr, total);
+          sm.big_appended = 1;
+        }
+        at = __shfl_sync(kFull, at, 31) + incl - mine;
+        const uint32_t slot = static_cast<uint32_t>(at >> 40);
+        if (big && slot < rc.big.cap) {
+          rc.big.e[slot] = make_uint4(beg, end, u, 0u);
+          rc.big.off[slot] = at & kBigEdgeMask;
+          wide = false;
+        }
+      }
+    }
+    for (unsigned m = __ballot_sync(kFull, wide); m; m &= m - 1) {
+      const int ld = __ffs(m) - 1;
+      const uint32_t wu = __shfl_sync(kFull, u, ld);
+      const uint32_t we = __shfl_sync(kFull, end, ld);
+      // a listed vertex that found the big list full walks its block edges here too
+      const uint32_t top = SH ? wu : (__shfl_sync(kFull, big ? 1u : 0u, ld) ? wu : lo);
+      uint32_t ru = wu - off;
+      for (uint32_t e = __shfl_sync(kFull, beg, ld) + lane; e < we; e += 32) {
+        const uint32_t v = ld_adj(p.col + e);
+        if (v < top && (!SH || v >= lo))
+          ru = uf_link<SH>(par, ru, uf_climb<SH>(par, v - off, uf_ld<SH>(par + (v - off))), hooked);
+      }
+    }
+  }
+}
+
+// Every vertex straight under its root. Two dependent reads per vertex, four
+// vertices in flight per thread.
+__device__ __forceinline__ void uf_flatten(const KParams& p) {
+  constexpr uint32_t U = 4;
+  const unsigned long long step = static_cast<unsigned long long>(gridDim.x) * kUfCta;
+  for (unsigned long long i = blockIdx.x * kUfCta + threadIdx.x; i < p.n; i += U * step) {
+    uint32_t f[U], x[U];
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) f[k] = i + k * step < p.n ? __ldca(p.state + (i + k * step)) : 0u;
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) x[k] = __ldca(p.state + f[k]);
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) {
+      if (x[k] == f[k] || i + k * step >= p.n) continue;
+      uint32_t r = x[k];
+      for (uint32_t y = __ldca(p.state + r); y != r; y = __ldca(p.state + r)) r = y;
+      __stcg(p.state + (i + k * step), r);
+    }
+  }
+}
+
+__device__ __forceinline__ void cc_jump_persistent(const KParams& p, Smem<kUfCta>& sm, uint32_t* tile) {
+  constexpr int CTA = kUfCta;
   init_smem<CTA>(sm);
   DevStatus* st = p.st;
   uint32_t gen = 0;
   const uint32_t ep0 = __ldcg(&st->epoch);
   if (p.skip_cta == static_cast<int>(blockIdx.x)) return;  // test hook: never arrives
   SingleView<OP_CCJ> g{p.row_ptr, p.col, p.w, p.state, p.stamp, p.n};
-  uint32_t edges = 0, dummy_t = 0, dummy_f = 0, rounds = 0, last_changes = 0;
-  fill_state<OP_CC>(p.state, p.n, nullptr, 0, blockIdx.x * CTA + threadIdx.x, gridDim.x * CTA);
+  const unsigned long long t_run0 = p.time_limit_ns ? globaltimer_ns() : 0ull;
+  uint32_t edges = 0, rounds = 0, hooks = 0, hooked = 0;
+  const uint32_t split = max(p.tn.cta_thresh, kUfSplit);
+  const uint32_t bs = uf_block_size(p.n, gridDim.x);
+  const uint32_t nblocks = p.n / bs + (p.n % bs != 0 ? 1u : 0u);
+  RoundCtx rc;
+  rc.out = Out{p.items[0], &st->tail[1], p.cap, &st->err};  // never pushed
+  rc.big = p.big;
+  rc.big_ctr = &st->big_ctr;
+  rc.limit = kInf;
+  rc.ds = nullptr;
+  rc.vis = nullptr;
+  rc.mf = nullptr;
+  rc.changes = &sm.round_pushes;  // the barrier publishes the grid's sum
+  for (uint32_t b = blockIdx.x; b < nblocks; b += gridDim.x) {
+    const uint32_t lo = b * bs, hi = lo + min(bs, p.n - lo);
+    for (uint32_t i = threadIdx.x; i < hi - lo; i += CTA) tile[i] = i;
+    __syncthreads();
+    uf_edges<true>(p, sm, rc, lo, hi, split, tile, edges, hooked);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < hi - lo; i += CTA) {
+      uint32_t x = tile[i];
+      for (uint32_t y = tile[x]; y != x; y = tile[x]) x = y;
+      __stcg(p.state + lo + i, lo + x);
+    }
+    __syncthreads();
+  }
+  if (hooked) atomicAdd(rc.changes, hooked);
   bool ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
-  trace_round(p.trace, p.trace_cap, 0, p.n, 0);
-  for (uint32_t r = 0; ok; ++r) {
-    RoundCtx rc;
-    rc.in_items = nullptr;  // every vertex
-    rc.in_n = p.n;
-    rc.out = Out{r & 1 ? p.items[0] : p.items[1], &st->tail[(r + 1) % 3], p.cap, &st->err};  // never pushed
-    rc.bfs_val = 0;
-    rc.ep = ep0 + r;
-    rc.grab = &st->grab[r % 3];
-    rc.tn = p.tn;
-    rc.big = p.big;
-    rc.big_ctr = &st->big_ctr;
-    rc.limit = kInf;
-    rc.far_out = Out{nullptr, nullptr, 0, &st->err};
-    rc.far_stamp = nullptr;
-    rc.phase = 0;
-    rc.changes = &sm.round_pushes;  // the barrier publishes the grid's sum
-    rc.mf = nullptr;
-    rc.row_ptr = p.row_ptr;
-    rc.vis = nullptr;
-    rc.ds = nullptr;
-    rc.dsr = 0;
-    rc.local_rounds = 0;
-    rc.local_items = nullptr;
+  hooks = sm.pub_out;
+  trace_round(p.trace, p.trace_cap, 0, p.n, hooks);
+  if (ok) {
     if (threadIdx.x == 0) {
-      if (blockIdx.x == 0) {
-        st->tail[(r + 2) % 3] = 0;
-        st->grab[(r + 2) % 3] = 0;
-      }
       sm.round_pushes = 0;
       sm.big_appended = 0;
     }
-    round_body<OP_CCJ, CTA, RED_NONE>(g, sm, rc, edges, dummy_t, dummy_f);
-    ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns, p.big.cap != 0);
-    if (!ok) break;
-    if (sm.pub_flags & kRelBigFlag) {
-      big_phase<OP_CCJ, CTA>(g, sm, rc, sm.pub_big);
-      ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
-      if (!ok) break;
-    }
-    last_changes = sm.pub_out;
-    // shortcut: every vertex points straight at its root
-    for (uint32_t v = blockIdx.x * CTA + threadIdx.x; v < p.n; v += gridDim.x * CTA) {
-      const uint32_t f0 = __ldcg(p.state + v);
-      uint32_t x = f0;
-      for (;;) {
-        const uint32_t y = __ldcg(p.state + x);
-        if (y == x) break;
-        x = y;
+    __syncthreads();
+    check_time_limit(&st->err, t_run0, p.time_limit_ns);
+    hooked = 0;
+    if (hooks < p.n / 2) {
+      // few edges stayed inside a block (ids without locality): link two neighbours
+      // of every vertex first and flatten, so that most of the edges below find both
+      // ends under one root and cost one read, instead of all racing to hook the
+      // same few roots (symmetric R-MAT, 2^16 vertices, 1.8 M entries: 142 us a call, the
+      // former kernel 311; 2^20, 31 M: 846, without this 770-1056, former 907-2421)
+      for (unsigned long long i = blockIdx.x * CTA + threadIdx.x; i < p.n; i += gridDim.x * CTA) {
+        const uint32_t u = static_cast<uint32_t>(i);
+        const uint32_t beg = __ldg(p.row_ptr + u), end = min(__ldg(p.row_ptr + u + 1), beg + 2u);
+        uint32_t ru = u;
+        for (uint32_t e = beg; e < end; ++e) {
+          const uint32_t v = __ldg(p.col + e);
+          if (v < p.n) ru = uf_link<false>(p.state, ru, uf_climb<false>(p.state, v, __ldca(p.state + v)), hooked);
+        }
       }
-      if (x != f0) __stcg(p.state + v, x);
+      if (hooked) atomicAdd(rc.changes, hooked);
+      hooked = 0;
+      ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
+      hooks |= sm.pub_out;
+      if (ok) {
+        uf_flatten(p);
+        if (threadIdx.x == 0) sm.round_pushes = 0;
+        ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
+      }
     }
-    ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
-    if (!ok) break;
-    rounds = r + 1;
-    trace_round(p.trace, p.trace_cap, rounds, p.n, last_changes);
-    if (last_changes == 0 || sm.pub_err != DERR_NONE) break;
-    if (rounds >= p.max_rounds) {
+  }
+  if (ok) {
+    if (threadIdx.x == 0) sm.round_pushes = 0;
+    __syncthreads();
+    for (uint32_t b = blockIdx.x; b < nblocks; b += gridDim.x)
+      uf_edges<false>(p, sm, rc, b * bs, b * bs + min(bs, p.n - b * bs), split, tile, edges, hooked);
+    if (hooked) atomicAdd(rc.changes, hooked);
+    ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns, p.big.cap != 0);
+    hooks |= sm.pub_out;
+    if (ok && (sm.pub_flags & kRelBigFlag)) {
+      const unsigned long long pub = sm.pub_big;
+      big_phase<OP_CCJ, CTA>(g, sm, rc, pub);
+      ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
+      hooks |= sm.pub_out;
+    }
+    if (ok) {
+      rounds = 1;
+      trace_round(p.trace, p.trace_cap, rounds, p.n, hooks);
+    }
+  }
+  if (ok && sm.pub_err == DERR_NONE && hooks != 0) {
+    if (p.max_rounds <= 1) {
       if (blockIdx.x == 0 && threadIdx.x == 0) set_err(&st->err, DERR_MAX_ROUNDS);
-      break;
+    } else {
+      uf_flatten(p);
+      rounds = 2;
+      trace_round(p.trace, p.trace_cap, rounds, p.n, 0);
     }
   }
   const unsigned long long esum = cta_sum_u64<CTA>(sm, edges);

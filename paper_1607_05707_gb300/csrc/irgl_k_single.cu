@@ -8,8 +8,14 @@ namespace irgl {
 template <uint32_t OP, int CTA>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_iterate(KParams p) {
   __shared__ Smem<CTA> sm;
-  if constexpr (OP == OP_CCJ) cc_jump_persistent<CTA>(p, sm);
-  else iterate_persistent<OP, CTA>(p, sm);
+  iterate_persistent<OP, CTA>(p, sm);
+}
+
+// Pointer-jumping CC: one CTA per SM, its vertex block in dynamic shared memory.
+__global__ void __launch_bounds__(kUfCta, 1) k_cc_jump(KParams p) {
+  __shared__ Smem<kUfCta> sm;
+  extern __shared__ uint32_t uf_tile[];
+  cc_jump_persistent(p, sm, uf_tile);
 }
 
 namespace {
@@ -38,6 +44,29 @@ cudaError_t launch_op(uint32_t cta, uint32_t grid, const KParams& p, cudaStream_
     case 1024: return launch_one<OP, 1024>(grid, p, s);
   }
   return cudaErrorInvalidValue;
+}
+
+constexpr size_t kUfBytes = sizeof(uint32_t) * kUfTile;
+
+cudaError_t occ_cc_jump(int* nb) {
+  // the opt-in size holds for later launches on this device
+  cudaError_t e = cudaFuncSetAttribute(k_cc_jump, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kUfBytes));
+  return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_cc_jump, kUfCta, kUfBytes);
+}
+
+cudaError_t launch_cc_jump(uint32_t cta, uint32_t grid, const KParams& p, cudaStream_t s) {
+  if (cta != static_cast<uint32_t>(kUfCta)) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kUfCta);
+  cfg.dynamicSmemBytes = kUfBytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_cc_jump, p);
 }
 
 // Resident CTAs per SM, after asking for the smallest shared-memory carveout
@@ -87,7 +116,7 @@ cudaError_t launch_iterate(uint32_t op, uint32_t cta, uint32_t grid, const KPara
     case OP_BFS: return launch_op<OP_BFS>(cta, grid, p, s);
     case OP_SSSP: return launch_op<OP_SSSP>(cta, grid, p, s);
     case OP_CC: return launch_op<OP_CC>(cta, grid, p, s);
-    case OP_CCJ: return launch_op<OP_CCJ>(cta, grid, p, s);
+    case OP_CCJ: return launch_cc_jump(cta, grid, p, s);
     case OP_BFSR: return launch_op<OP_BFSR>(cta, grid, p, s);
   }
   return cudaErrorInvalidValue;
@@ -98,7 +127,7 @@ cudaError_t occupancy_iterate(uint32_t op, uint32_t cta, int* nb) {
     case OP_BFS: return occ_op<OP_BFS>(cta, nb);
     case OP_SSSP: return occ_op<OP_SSSP>(cta, nb);
     case OP_CC: return occ_op<OP_CC>(cta, nb);
-    case OP_CCJ: return occ_op<OP_CCJ>(cta, nb);
+    case OP_CCJ: return occ_cc_jump(nb);
     case OP_BFSR: return occ_op<OP_BFSR>(cta, nb);
   }
   return cudaErrorInvalidValue;
