@@ -33,7 +33,7 @@ struct irgl_ctx {
   uint32_t ws_far_n = 0;
   uint32_t* ws_stamp = nullptr;  // SSSP/CC push dedup stamps
   uint32_t ws_stamp_n = 0;
-  uint32_t* msf_buf = nullptr;   // minimum spanning forest workspace (status block + 14 arrays of msf_n)
+  uint32_t* msf_buf = nullptr;   // minimum spanning forest workspace (status block + 16 arrays of msf_n)
   uint32_t msf_n = 0;
   void* msf_host = nullptr;      // pinned copy of its status block
   uint32_t* ws_bu[2] = {nullptr, nullptr};  // direction-optimising BFS: open-vertex lists

@@ -23,9 +23,19 @@
 //                       find_min is invoked again on that list, with contiguous
 //                       blocks of items per thread (Retry Backoff), until it is
 //                       empty.
-// Before taking a lock a thread compares its weight with the component's
-// current one (weights only fall within an iteration), so most vertices never
-// lock.
+// Before taking a lock a thread lowers the component's (w, min(u,v)) prefix with
+// one 64-bit atomicMin; only a thread that lowered (or tied) it enters the Atomic
+// section, and there only the owner of the current prefix writes, so of k threads
+// that meet at a component about ln k lock instead of every one that saw no record
+// yet.
+//
+// What bounds it: the live vertices' adjacency and the parent of each neighbour
+// once per iteration, and a 32-byte record per component, one sector for prefix,
+// lock and fields (six arrays before). The lists (vertices, components, retries,
+// edges) are staged in shared memory and appended by one atomic per few hundred
+// items: one atomic per component on single counters was a third of the time
+// (2048^2 mesh, retry locks: link of the first iteration 2.03 ms of 6.4; now 2.0 ms in
+// all; blocking and ticket locks 14.7 and 13.0 -> 1.97 and 1.93 ms).
 //
 // Outlined (IRGL_PERSISTENT): the three kernels run back to back in one
 // cooperative launch, separated by the grid barrier; the CTA size is chosen by
@@ -67,19 +77,29 @@ struct MsfStatus {
 };
 static_assert(sizeof(MsfStatus) % 128 == 0, "status layout");
 
+constexpr unsigned long long kNoRecord = ~0ull;
+
+// A component's lightest cross edge, one 32-byte sector. wl is lowered by
+// atomicMin before the lock is taken; tag is the prefix that hi, e and other
+// belong to (written inside the Atomic section).
+struct __align__(32) MsfRec {
+  unsigned long long wl;   // (w << 32) | min(u,v) of the lightest edge found (~0: none yet)
+  unsigned long long tag;  // prefix of the edge described below
+  uint32_t hi;             // its larger endpoint
+  uint32_t e;              // its CSR index
+  uint32_t other;          // the component at its other end
+  uint32_t lock;           // 0/1 (BLOCKING, RETRY) or now-serving (TICKET)
+};
+static_assert(sizeof(MsfRec) == 32, "one sector");
+
 struct MsfParams {
   const uint32_t* __restrict__ row_ptr;
   const uint32_t* __restrict__ col;
   const int32_t* __restrict__ w;
   uint32_t n;
   uint32_t* comp;    // component (root vertex) of each vertex
-  unsigned long long* cwl;  // per component: lightest cross edge's (w << 32) | min(u,v) (~0: none yet),
-                            // one word so the pre-lock test reads a consistent prefix of the key
-  uint32_t* chi;     //   its larger endpoint
-  uint32_t* cedge;   //   its CSR index
-  uint32_t* cother;  //   the component at its other end
-  uint32_t* lock;    // per component: 0/1 (BLOCKING, RETRY) or now-serving (TICKET)
-  uint32_t* ticket;  // per component: next ticket (TICKET)
+  struct MsfRec* rec;  // per component
+  uint32_t* ticket;    // per component: next ticket (TICKET)
   uint32_t* items[2];  // in/out worklists of vertices (capacity n each)
   uint32_t* retry[2];  // retry worklists (capacity n each)
   uint32_t* comps;     // components with a record this iteration (capacity n)
@@ -108,16 +128,25 @@ struct MinEdge {
 __device__ __forceinline__ MinEdge no_edge() { return MinEdge{kInf, kInf, kInf, 0u, 0u}; }
 
 // Lightest cross-component edge among u's edges [beg, end), lanes taking
-// every stride-th edge from beg + rank.
+// every stride-th edge from beg + rank, four columns, components and weights in
+// flight.
 __device__ __forceinline__ void scan_edges(const MsfParams& p, uint32_t u, uint32_t cu, uint32_t beg, uint32_t end,
                                            uint32_t rank, uint32_t stride, MinEdge& best) {
-  for (uint32_t e = beg + rank; e < end; e += stride) {
-    const uint32_t v = __ldg(p.col + e);
-    const uint32_t cv = __ldcg(p.comp + v);
-    if (cv == cu) continue;
-    const uint32_t wt = static_cast<uint32_t>(__ldg(p.w + e));
-    const uint32_t lo = min(u, v), hi = max(u, v);
-    if (key_less(wt, lo, hi, best.w, best.lo, best.hi)) best = MinEdge{wt, lo, hi, e, cv};
+  for (unsigned long long e0 = static_cast<unsigned long long>(beg) + rank; e0 < end; e0 += 4ull * stride) {
+    uint32_t v[4], cv[4], wt[4];
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) v[k] = e0 + k * stride < end ? __ldg(p.col + e0 + k * stride) : u;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) cv[k] = v[k] != u ? __ldcg(p.comp + v[k]) : cu;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) wt[k] = cv[k] != cu ? static_cast<uint32_t>(__ldg(p.w + e0 + k * stride)) : kInf;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      if (cv[k] == cu) continue;
+      const uint32_t lo = min(u, v[k]), hi = max(u, v[k]);
+      if (key_less(wt[k], lo, hi, best.w, best.lo, best.hi))
+        best = MinEdge{wt[k], lo, hi, static_cast<uint32_t>(e0) + k * stride, cv[k]};
+    }
   }
 }
 
@@ -135,69 +164,104 @@ __device__ __forceinline__ MinEdge warp_min_edge(MinEdge b) {
   return b;
 }
 
-// Warp-aggregated push of `item` (where pred) to list[base + ...], counting in *ctr.
-__device__ __forceinline__ void warp_push(uint32_t* list, uint32_t base, uint32_t cap, uint32_t* ctr, bool pred,
-                                          uint32_t item, uint32_t* err) {
+// Three lists staged in the CTA's shared stage (L: vertices or edges, components,
+// retries). Each thread pushes at most one item per list and tile; the stage is
+// flushed at CTA-uniform points once a list might not hold another tile, with one
+// atomic on the list's counter and coalesced stores.
+template <int CTA>
+struct MsfLists {
+  static constexpr uint32_t kCap = (Smem<CTA>::kStage / 3) & ~31u;
+  static_assert(kCap >= 2 * CTA, "room for the tile that follows the flush test");
+  uint32_t n[3];
+  uint32_t at[3];
+};
+
+template <int CTA>
+__device__ __forceinline__ void stage_item(Smem<CTA>& sm, MsfLists<CTA>& ls, uint32_t L, bool pred, uint32_t item) {
   const unsigned m = __ballot_sync(kFull, pred);
   if (m == 0) return;
   const uint32_t lane = threadIdx.x & 31;
   const int leader = __ffs(m) - 1;
   uint32_t pos = 0;
-  if (lane == static_cast<uint32_t>(leader)) pos = atomicAdd(ctr, static_cast<uint32_t>(__popc(m)));
+  if (lane == static_cast<uint32_t>(leader)) pos = atomicAdd(&ls.n[L], static_cast<uint32_t>(__popc(m)));
   pos = __shfl_sync(kFull, pos, leader) + __popc(m & lanemask_lt());
-  if (pred) {
-    if (base + pos < cap) __stcg(list + base + pos, item);
-    else set_err(err, DERR_WL_OVERFLOW);
-  }
+  if (pred) sm.stage[L * MsfLists<CTA>::kCap + pos] = item;
 }
 
-constexpr unsigned long long kNoRecord = ~0ull;
+// Append the staged items: list L to dst[L][base[L] + ...] (capacity cap[L]), counted in *ctr[L].
+struct MsfDest {
+  uint32_t* dst[3];
+  uint32_t* ctr[3];
+  uint32_t base[3];
+  uint32_t cap[3];
+};
+template <int CTA>
+__device__ __forceinline__ void flush_lists(Smem<CTA>& sm, MsfLists<CTA>& ls, const MsfDest& d, uint32_t above,
+                                            uint32_t* err) {
+  constexpr uint32_t C = MsfLists<CTA>::kCap;
+  if (!__syncthreads_or(ls.n[0] > above || ls.n[1] > above || ls.n[2] > above)) return;
+  if (threadIdx.x < 3 && ls.n[threadIdx.x] != 0) {
+    const uint32_t L = threadIdx.x;
+    uint32_t* const ctr = L == 0 ? d.ctr[0] : L == 1 ? d.ctr[1] : d.ctr[2];
+    ls.at[L] = (L == 0 ? d.base[0] : L == 1 ? d.base[1] : d.base[2]) + atomicAdd(ctr, ls.n[L]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (uint32_t L = 0; L < 3; ++L) {
+    const uint32_t k = ls.n[L], at = ls.at[L];
+    for (uint32_t i = threadIdx.x; i < k; i += CTA) {
+      if (at + i < d.cap[L]) __stcg(d.dst[L] + at + i, sm.stage[L * C + i]);
+      else set_err(err, DERR_WL_OVERFLOW);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) ls.n[threadIdx.x] = 0;
+  __syncthreads();
+}
 
 __device__ __forceinline__ unsigned long long wl_of(const MinEdge& k) {
   return (static_cast<unsigned long long>(k.w) << 32) | k.lo;
 }
 
-// The critical section of the Atomic: keep the lighter of the component's
-// record and this edge. The first edge of the iteration lists the component.
-__device__ __forceinline__ void record_update(const MsfParams& p, uint32_t c, const MinEdge& k, MsfSlot* slot,
-                                              uint32_t comp_base) {
-  const unsigned long long wl0 = __ldcg(p.cwl + c), wl = wl_of(k);
-  if (wl > wl0 || (wl == wl0 && k.hi >= __ldcg(p.chi + c))) return;
-  if (wl0 == kNoRecord) {
-    const uint32_t pos = comp_base + atomicAdd(&slot->comp, 1u);
-    if (pos < p.n) __stcg(p.comps + pos, c);
-    else set_err(&p.st->err, DERR_WL_OVERFLOW);
-  }
-  __stcg(p.cwl + c, wl);
-  __stcg(p.chi + c, k.hi);
-  __stcg(p.cedge + c, k.e);
-  __stcg(p.cother + c, k.other);
+// The critical section of the Atomic: the owner of the component's current
+// prefix describes its edge; of equal prefixes the smaller larger end stays.
+__device__ __forceinline__ void record_update(MsfRec* r, const MinEdge& k) {
+  const unsigned long long wl = wl_of(k);
+  const ulonglong2 cur = __ldcg(reinterpret_cast<const ulonglong2*>(r));  // wl, tag
+  if (cur.x != wl || (cur.y == wl && k.hi >= __ldcg(&r->hi))) return;
+  __stcg(&r->tag, wl);
+  __stcg(reinterpret_cast<uint2*>(&r->hi), make_uint2(k.hi, k.e));
+  __stcg(&r->other, k.other);
 }
 
 __device__ __forceinline__ unsigned long long msf_now() { return globaltimer_ns(); }
 
 // Atomic(lock[c]) { record_update } in the configured form. Returns false when
-// the lock was missed in RETRY mode (the caller retries the vertex).
-__device__ __forceinline__ bool atomic_update(const MsfParams& p, uint32_t c, const MinEdge& k, MsfSlot* slot,
-                                              uint32_t comp_base) {
-  // test before locking: the record only gets lighter within an iteration, and
-  // its (w, lo) prefix is one word, so a heavier prefix can never win
-  if (wl_of(k) > __ldcg(p.cwl + c)) return true;
+// the lock was missed in RETRY mode (the caller retries the vertex). first: this
+// edge is the component's first of the iteration; locks counts acquisitions.
+__device__ __forceinline__ bool atomic_update(const MsfParams& p, uint32_t c, const MinEdge& k, bool& first,
+                                              uint32_t& locks) {
+  MsfRec* const r = p.rec + c;
+  const unsigned long long wl = wl_of(k);
+  if (wl > __ldcg(&r->wl)) return true;
+  const unsigned long long before = atomicMin(&r->wl, wl);
+  if (before < wl) return true;
+  first = before == kNoRecord;
   if (p.lock_mode == IRGL_LOCK_TICKET) {
     const uint32_t t = atomicAdd(p.ticket + c, 1u);
     const unsigned long long t0 = msf_now();
     for (uint32_t spins = 1;; ++spins) {
       uint32_t serving;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(serving) : "l"(p.lock + c) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(serving) : "l"(&r->lock) : "memory");
       if (serving == t) break;
       if ((spins & 63u) == 0 && (msf_now() - t0 > p.lock_timeout_ns || __ldcg(&p.st->err) == DERR_LOCK_TIMEOUT)) {
         set_err(&p.st->err, DERR_LOCK_TIMEOUT);
         return true;
       }
     }
-    record_update(p, c, k, slot, comp_base);
-    atomicAdd(&p.ms->locks, 1u);
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" : : "l"(p.lock + c), "r"(t + 1u) : "memory");
+    record_update(r, k);
+    ++locks;
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" : : "l"(&r->lock), "r"(t + 1u) : "memory");
     return true;
   }
   const bool blocking = p.lock_mode == IRGL_LOCK_BLOCKING;
@@ -206,11 +270,11 @@ __device__ __forceinline__ bool atomic_update(const MsfParams& p, uint32_t c, co
     // the attempt and the critical section in one branch: no thread waits on
     // a lock held by a lane of its own warp that cannot be scheduled
     uint32_t old;
-    asm volatile("atom.acquire.gpu.global.cas.b32 %0, [%1], 0, 1;" : "=r"(old) : "l"(p.lock + c) : "memory");
+    asm volatile("atom.acquire.gpu.global.cas.b32 %0, [%1], 0, 1;" : "=r"(old) : "l"(&r->lock) : "memory");
     if (old == 0u) {
-      record_update(p, c, k, slot, comp_base);
-      atomicAdd(&p.ms->locks, 1u);
-      asm volatile("st.release.gpu.global.u32 [%0], 0;" : : "l"(p.lock + c) : "memory");
+      record_update(r, k);
+      ++locks;
+      asm volatile("st.release.gpu.global.u32 [%0], 0;" : : "l"(&r->lock) : "memory");
       return true;
     }
     if (!blocking) return false;  // Atomic ... Else: Retry
@@ -226,7 +290,7 @@ __device__ __forceinline__ bool atomic_update(const MsfParams& p, uint32_t c, co
 // their edges to the Atomic section (the others cannot change the record).
 // Returns true when that lane missed the lock in RETRY mode.
 __device__ __forceinline__ bool aggregate_update(const MsfParams& p, bool found, uint32_t cu, const MinEdge& best,
-                                                 MsfSlot* slot, uint32_t comp_base) {
+                                                 bool& first, uint32_t& locks) {
   const unsigned active = __ballot_sync(kFull, found);
   if (!found) return false;
   const unsigned peers = __match_any_sync(active, cu);
@@ -234,56 +298,39 @@ __device__ __forceinline__ bool aggregate_update(const MsfParams& p, bool found,
   const uint32_t ml = __reduce_min_sync(peers, best.w == mw ? best.lo : kInf);
   const uint32_t mh = __reduce_min_sync(peers, best.w == mw && best.lo == ml ? best.hi : kInf);
   if (best.w != mw || best.lo != ml || best.hi != mh) return false;
-  return !atomic_update(p, cu, best, slot, comp_base);
+  return !atomic_update(p, cu, best, first, locks);
 }
 
 // find_min over a worklist: `in` (nullptr = vertices 0..in_n-1). Default
 // mapping: a warp takes 32 consecutive items; lists of 32 edges or more are
 // scanned by the whole warp. Retry mapping (Retry Backoff): thread t takes the
-// contiguous block [t * B, (t + 1) * B) and scans each list alone.
-__device__ void msf_find_min(const MsfParams& p, const uint32_t* in, uint32_t in_n, bool backoff, uint32_t* out,
-                             uint32_t out_base, uint32_t* retry_out, MsfSlot* slot, uint32_t comp_base,
-                             uint32_t gtid, uint32_t nthreads) {
+// contiguous block [t * B, (t + 1) * B) and scans each list alone. Trip counts
+// are CTA-uniform (the lists are flushed by the whole CTA).
+template <int CTA>
+__device__ void msf_find_min(const MsfParams& p, Smem<CTA>& sm, MsfLists<CTA>& ls, const uint32_t* in, uint32_t in_n,
+                             bool backoff, uint32_t* out, uint32_t out_base, uint32_t* retry_out, MsfSlot* slot,
+                             uint32_t comp_base) {
   const uint32_t lane = threadIdx.x & 31;
-  if (backoff) {
-    const uint32_t B = (in_n + nthreads - 1) / nthreads;
-    const uint32_t lo = min(gtid * B, in_n), hi = min(lo + B, in_n);
-    // warp-uniform trip count so the warp-aggregated pushes see converged warps
-    uint32_t trips = hi - lo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) trips = max(trips, __shfl_xor_sync(kFull, trips, o));
-    for (uint32_t t = 0; t < trips; ++t) {
-      const uint32_t i = lo + t;
-      const bool valid = i < hi;
-      uint32_t u = 0, cu = 0;
-      bool found = false, missed = false;
-      MinEdge best = no_edge();
-      if (valid) {
-        u = __ldcg(in + i);
-        cu = __ldcg(p.comp + u);
-        best = no_edge();
-        scan_edges(p, u, cu, __ldg(p.row_ptr + u), __ldg(p.row_ptr + u + 1), 0, 1, best);
-        found = best.w != kInf;
-      }
-      missed = aggregate_update(p, found, cu, best, slot, comp_base);
-      warp_push(out, out_base, p.n, &slot->out, found && !missed, u, &p.st->err);
-      warp_push(retry_out, 0, p.n, &slot->retry, missed, u, &p.st->err);
-    }
-    return;
-  }
-  const uint32_t wid = gtid >> 5, nwarps = nthreads >> 5;
-  for (uint32_t base = wid * 32; base < in_n; base += nwarps * 32) {
-    const uint32_t idx = base + lane;
+  const uint32_t gtid = blockIdx.x * CTA + threadIdx.x, nthreads = gridDim.x * CTA;
+  constexpr uint32_t kFlush = MsfLists<CTA>::kCap - CTA;
+  const MsfDest d{{out, p.comps, retry_out}, {&slot->out, &slot->comp, &slot->retry}, {out_base, comp_base, 0u}, {p.n, p.n, p.n}};
+  uint32_t locks = 0;
+  const uint32_t trips = backoff ? (in_n + nthreads - 1) / nthreads
+                                 : static_cast<uint32_t>((static_cast<unsigned long long>(in_n) + nthreads - 1u -
+                                                          min(in_n, blockIdx.x * CTA)) / nthreads);
+  for (uint32_t t = 0; t < trips; ++t) {
+    const unsigned long long idx = backoff ? static_cast<unsigned long long>(gtid) * trips + t
+                                           : static_cast<unsigned long long>(t) * nthreads + gtid;
     const bool valid = idx < in_n;
     uint32_t u = 0, cu = 0, beg = 0, end = 0;
     if (valid) {
-      u = in ? __ldcg(in + idx) : idx;
+      u = in ? __ldcg(in + idx) : static_cast<uint32_t>(idx);
       cu = __ldcg(p.comp + u);
       beg = __ldg(p.row_ptr + u);
       end = __ldg(p.row_ptr + u + 1);
     }
     MinEdge best = no_edge();
-    const bool big = valid && end - beg >= 32u;
+    const bool big = !backoff && valid && end - beg >= 32u;
     if (valid && !big) scan_edges(p, u, cu, beg, end, 0, 1, best);
     for (unsigned m = __ballot_sync(kFull, big); m; m &= m - 1) {
       const int l = __ffs(m) - 1;
@@ -294,51 +341,99 @@ __device__ void msf_find_min(const MsfParams& p, const uint32_t* in, uint32_t in
       if (lane == static_cast<uint32_t>(l)) best = wb;
     }
     const bool found = best.w != kInf;
-    const bool missed = aggregate_update(p, found, cu, best, slot, comp_base);
-    warp_push(out, out_base, p.n, &slot->out, found && !missed, u, &p.st->err);
-    warp_push(retry_out, 0, p.n, &slot->retry, missed, u, &p.st->err);
+    bool first = false;
+    const bool missed = aggregate_update(p, found, cu, best, first, locks);
+    __syncwarp();
+    stage_item<CTA>(sm, ls, 0, found && !missed, u);
+    stage_item<CTA>(sm, ls, 1, first, cu);
+    stage_item<CTA>(sm, ls, 2, missed, u);
+    flush_lists<CTA>(sm, ls, d, kFlush, &p.st->err);
   }
+  flush_lists<CTA>(sm, ls, d, 0u, &p.st->err);
+  locks = __reduce_add_sync(kFull, locks);
+  if (lane == 0 && locks) atomicAdd(&p.ms->locks, locks);
 }
 
 // link over the components with a record: record the edge (once per mutual
 // pair: by the smaller component) and hook the component to the other one
 // (a mutual pair's smaller component stays the root), then clear the record.
-__device__ void msf_link(const MsfParams& p, uint32_t comp_n, uint32_t gtid, uint32_t nthreads) {
-  for (uint32_t i = gtid; i < comp_n; i += nthreads) {
-    const uint32_t c = __ldcg(p.comps + i);
-    const uint32_t c2 = __ldcg(p.cother + c);
-    const bool mutual = __ldcg(p.cother + c2) == c;
-    if (!mutual || c < c2) {
-      const uint32_t pos = atomicAdd(&p.ms->edges, 1u);
-      if (pos < p.out_cap) __stcg(p.out_edges + pos, __ldcg(p.cedge + c));
-      else set_err(&p.st->err, DERR_WL_OVERFLOW);
-      atomicAdd(&p.ms->weight, __ldcg(p.cwl + c) >> 32);
+// The forest's edges go through the stage, its weight is summed per warp.
+template <int CTA>
+__device__ void msf_link(const MsfParams& p, Smem<CTA>& sm, MsfLists<CTA>& ls, uint32_t comp_n) {
+  const uint32_t gtid = blockIdx.x * CTA + threadIdx.x, nthreads = gridDim.x * CTA;
+  constexpr uint32_t kFlush = MsfLists<CTA>::kCap - CTA;
+  const MsfDest d{{p.out_edges, nullptr, nullptr}, {&p.ms->edges, nullptr, nullptr}, {0u, 0u, 0u}, {p.out_cap, 0u, 0u}};
+  unsigned long long weight = 0;
+  const uint32_t trips = static_cast<uint32_t>((static_cast<unsigned long long>(comp_n) + nthreads - 1u -
+                                                min(comp_n, blockIdx.x * CTA)) / nthreads);
+  for (uint32_t t = 0; t < trips; ++t) {
+    const unsigned long long i = static_cast<unsigned long long>(t) * nthreads + gtid;
+    bool take = false;
+    uint32_t edge = 0;
+    if (i < comp_n) {
+      const uint32_t c = __ldcg(p.comps + i);
+      MsfRec* const r = p.rec + c;
+      const uint4 f = __ldcg(reinterpret_cast<const uint4*>(&r->hi));  // hi, e, other, lock
+      const uint32_t w = static_cast<uint32_t>(__ldcg(&r->wl) >> 32);
+      const uint32_t c2 = f.z;
+      const bool mutual = __ldcg(&p.rec[c2].other) == c;
+      take = !mutual || c < c2;
+      edge = f.y;
+      if (take) weight += w;
+      if (!mutual || c > c2) __stcg(p.comp + c, c2);
+      __stcg(reinterpret_cast<ulonglong2*>(r), make_ulonglong2(kNoRecord, kNoRecord));
     }
-    if (!mutual || c > c2) __stcg(p.comp + c, c2);
-    __stcg(p.cwl + c, kNoRecord);
+    stage_item<CTA>(sm, ls, 0, take, edge);
+    flush_lists<CTA>(sm, ls, d, kFlush, &p.st->err);
   }
+  flush_lists<CTA>(sm, ls, d, 0u, &p.st->err);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) weight += __shfl_xor_sync(kFull, weight, o);
+  if ((threadIdx.x & 31) == 0 && weight) atomicAdd(&p.ms->weight, weight);
 }
 
-// One pointer-jumping pass over every vertex; returns this thread's updates.
+// One pointer-jumping pass over every vertex: each follows its pointers to the
+// root, kJumpSteps at most, four vertices in flight per thread. Returns how many
+// stopped short of a root (the pass is repeated while any did): a hooked tree is
+// rarely deeper, so one pass does what took four or five of one step each, and a
+// long chain still shrinks by more than kJumpSteps a pass.
+constexpr uint32_t kJumpSteps = 64;
 __device__ uint32_t msf_jump(const MsfParams& p, uint32_t gtid, uint32_t nthreads) {
-  uint32_t changed = 0;
-  for (uint32_t v = gtid; v < p.n; v += nthreads) {
-    const uint32_t c = __ldcg(p.comp + v);
-    const uint32_t cc = __ldcg(p.comp + c);
-    if (cc != c) {
-      __stcg(p.comp + v, cc);
-      ++changed;
+  constexpr uint32_t U = 4;
+  uint32_t open = 0;
+  for (unsigned long long i = gtid; i < p.n; i += static_cast<unsigned long long>(U) * nthreads) {
+    uint32_t c[U], x[U];
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) {
+      const unsigned long long v = i + static_cast<unsigned long long>(k) * nthreads;
+      c[k] = v < p.n ? __ldcg(p.comp + v) : 0u;
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) x[k] = __ldcg(p.comp + c[k]);
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) {
+      const unsigned long long v = i + static_cast<unsigned long long>(k) * nthreads;
+      if (v >= p.n || x[k] == c[k]) continue;
+      uint32_t r = x[k], y = __ldcg(p.comp + r);
+      for (uint32_t s = 2; y != r && s < kJumpSteps; ++s) {
+        r = y;
+        y = __ldcg(p.comp + r);
+      }
+      open += y != r ? 1u : 0u;
+      __stcg(p.comp + v, r);
     }
   }
-  return changed;
+  return open;
 }
 
 __device__ void msf_init(const MsfParams& p, uint32_t gtid, uint32_t nthreads) {
-  for (uint32_t v = gtid; v < p.n; v += nthreads) {
+  for (unsigned long long i = gtid; i < p.n; i += nthreads) {
+    const uint32_t v = static_cast<uint32_t>(i);
     __stcg(p.comp + v, v);
-    __stcg(p.cwl + v, kNoRecord);
     // a held lock: 1 for the CAS forms, a now-serving value no ticket reaches
-    __stcg(p.lock + v, v == p.held_lock ? (p.ticket ? kInf : 1u) : 0u);
+    const uint32_t lock = v == p.held_lock ? (p.ticket ? kInf : 1u) : 0u;
+    __stcg(reinterpret_cast<ulonglong2*>(p.rec + v), make_ulonglong2(kNoRecord, kNoRecord));
+    __stcg(reinterpret_cast<uint4*>(&p.rec[v].hi), make_uint4(0u, 0u, 0u, lock));
     if (p.ticket) __stcg(p.ticket + v, 0u);
   }
 }
@@ -354,6 +449,8 @@ __device__ __forceinline__ uint32_t cta_sum_u32(Smem<CTA>& sm, uint32_t x) {
 template <int CTA>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_msf(MsfParams p) {
   __shared__ Smem<CTA> sm;
+  __shared__ MsfLists<CTA> ls;
+  if (threadIdx.x < 3) ls.n[threadIdx.x] = 0;
   init_smem<CTA>(sm);
   DevStatus* st = p.st;
   MsfStatus* ms = p.ms;
@@ -403,8 +500,7 @@ __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_msf(MsfParams p)
     const unsigned long long t_retry0 = msf_now();
     for (;;) {
       begin_invocation();
-      msf_find_min(p, fin, fin_n, backoff, out, out_total, p.retry[rb], &ms->slot[inv % 3], comp_total, gtid,
-                   nthreads);
+      msf_find_min<CTA>(p, sm, ls, fin, fin_n, backoff, out, out_total, p.retry[rb], &ms->slot[inv % 3], comp_total);
       const MsfSlot s = end_invocation();
       if (!ok) break;
       out_total += s.out;
@@ -421,7 +517,7 @@ __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_msf(MsfParams p)
     }
     if (!ok || out_total == 0) break;  // no component has a cross edge: the forest is complete
     begin_invocation();
-    msf_link(p, min(comp_total, p.n), gtid, nthreads);
+    msf_link<CTA>(p, sm, ls, min(comp_total, p.n));
     end_invocation();
     for (uint32_t pass = 0; ok; ++pass) {
       begin_invocation();
@@ -462,16 +558,20 @@ struct MsfStep {
 
 template <int CTA>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_msf_step(MsfParams p, MsfStep s) {
+  __shared__ Smem<CTA> sm;
+  __shared__ MsfLists<CTA> ls;
+  if (threadIdx.x < 3) ls.n[threadIdx.x] = 0;
+  __syncthreads();
   const uint32_t gtid = blockIdx.x * CTA + threadIdx.x, nthreads = gridDim.x * CTA;
   MsfSlot* slot = &p.ms->slot[s.slot];
   switch (s.phase) {
     case MSF_INIT: msf_init(p, gtid, nthreads); break;
     case MSF_FIND:
     case MSF_FIND_RETRY:
-      msf_find_min(p, s.in, s.in_n, s.phase == MSF_FIND_RETRY, s.out, s.out_base, s.retry_out, slot, s.comp_base, gtid,
-                   nthreads);
+      msf_find_min<CTA>(p, sm, ls, s.in, s.in_n, s.phase == MSF_FIND_RETRY, s.out, s.out_base, s.retry_out, slot,
+                        s.comp_base);
       break;
-    case MSF_LINK: msf_link(p, s.comp_n, gtid, nthreads); break;
+    case MSF_LINK: msf_link<CTA>(p, sm, ls, s.comp_n); break;
     case MSF_JUMP: {
       const uint32_t c = msf_jump(p, gtid, nthreads);
       if (c) atomicAdd(&slot->changed, c);
@@ -567,8 +667,8 @@ irgl_status irgl_msf(irgl_ctx* ctx, irgl_graph* g, irgl_mode mode, irgl_lock loc
   s = control_cta(masks, 3, t.cta_size, &cta);
   if (s != IRGL_OK) return s;
 
-  // workspace: the status block, then 14 arrays of N words (N a multiple of
-  // 64, so every array starts on a 256-byte boundary; cwl takes two)
+  // workspace: the status block, then 16 arrays of N words (N a multiple of
+  // 64, so every array starts on a 256-byte boundary; the records take eight)
   const uint64_t n_round = (static_cast<uint64_t>(n) + 63u) & ~63ull;
   if (n_round > 0xFFFFFFC0ull) return fail(IRGL_ERR_INVALID_ARG, "n = %u is too large for the forest workspace", n);
   if (ctx->msf_n < n_round || !ctx->msf_buf) {
@@ -576,7 +676,7 @@ irgl_status irgl_msf(irgl_ctx* ctx, irgl_graph* g, irgl_mode mode, irgl_lock loc
     cudaFree(ctx->msf_buf);
     ctx->msf_buf = nullptr;
     ctx->msf_n = 0;
-    const size_t words = static_cast<size_t>(n_round) * 14 + sizeof(MsfStatus) / 4;
+    const size_t words = static_cast<size_t>(n_round) * 16 + sizeof(MsfStatus) / 4;
     cudaError_t e = cudaMalloc(&ctx->msf_buf, words * sizeof(uint32_t));
     if (e != cudaSuccess) return cuda_fail(e, "minimum spanning forest workspace");
     ctx->msf_n = static_cast<uint32_t>(n_round);
@@ -595,19 +695,15 @@ irgl_status irgl_msf(irgl_ctx* ctx, irgl_graph* g, irgl_mode mode, irgl_lock loc
   p.n = n;
   MsfStatus* ms = reinterpret_cast<MsfStatus*>(b);  // 128-byte multiple at the start
   uint32_t* a = b + sizeof(MsfStatus) / 4;
-  p.comp = a + 0 * N;
-  p.cwl = reinterpret_cast<unsigned long long*>(a + 1 * N);  // two arrays' worth
-  p.chi = a + 3 * N;
-  p.cedge = a + 4 * N;
-  p.cother = a + 5 * N;
-  p.lock = a + 6 * N;
-  p.ticket = lock == IRGL_LOCK_TICKET ? a + 7 * N : nullptr;
-  p.items[0] = a + 8 * N;
-  p.items[1] = a + 9 * N;
-  p.retry[0] = a + 10 * N;
-  p.retry[1] = a + 11 * N;
-  p.comps = a + 12 * N;
-  uint32_t* dev_out = out_on_host ? a + 13 * N : out_edges;
+  p.rec = reinterpret_cast<MsfRec*>(a);  // eight arrays' worth
+  p.comp = a + 8 * N;
+  p.ticket = lock == IRGL_LOCK_TICKET ? a + 9 * N : nullptr;
+  p.items[0] = a + 10 * N;
+  p.items[1] = a + 11 * N;
+  p.retry[0] = a + 12 * N;
+  p.retry[1] = a + 13 * N;
+  p.comps = a + 14 * N;
+  uint32_t* dev_out = out_on_host ? a + 15 * N : out_edges;
   p.out_edges = dev_out;
   p.out_cap = out_on_host ? n : cap;
   p.lock_mode = static_cast<uint32_t>(lock);
