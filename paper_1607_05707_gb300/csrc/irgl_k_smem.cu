@@ -13,6 +13,15 @@
 // each round) and fixed point as the grid-wide kernels; only the schedule of
 // the pops differs, which the unique fixed point does not see.
 //
+// What bounds it: the round's chain of dependent shared-memory reads and atomics
+// (about 30 and 100 cycles each) and its barrier. So a round has one barrier (three
+// list counters in turn), a warp's pushes one atomic, and a frontier of up to 256
+// items gives every item four lanes, dealt across the warps; larger ones have their
+// edges dealt to the lanes by a scan. 64 x 64 grid BFS, 113 rounds: 1.1 us a round
+// and 128 us a call before, 0.65 and 99.5 us now; R-MAT of 2^10 vertices, SSSP: 97
+// -> 62 us (rounds of 360-525 items 5-10 us before, and 13 us went to 1024 threads
+// adding their edge counts to one 64-bit word).
+//
 // Shared-memory layout (32-bit words): row_ptr[n + 1], col[m], w[m] (SSSP),
 // value[n], stamp[n] (SSSP and CC: the round that last pushed the vertex, so
 // each vertex is pushed at most once per round), wl[2][n].
@@ -25,35 +34,38 @@ namespace irgl {
 namespace {
 
 constexpr int kSmemCta = 1024;
+constexpr uint32_t kSmemWarps = kSmemCta / 32;
+constexpr uint32_t kSmemFour = kSmemCta / 4;  // frontiers of at most this many items give each four lanes
 constexpr uint32_t kInitMark = 0xFFFFFFFEu;  // stamp of the round-0 items (CC)
 
-template <uint32_t OP>
-__device__ __forceinline__ void smem_push(uint32_t* out, uint32_t* out_n, uint32_t cap, uint32_t v, uint32_t* err) {
-  const uint32_t pos = atomicAdd(out_n, 1u);
-  if (pos < cap) out[pos] = v;
-  else atomicCAS(err, DERR_NONE, DERR_WL_OVERFLOW);
+// Warp-aggregated push: one shared atomic per warp that pushes anything.
+__device__ __forceinline__ void smem_push(uint32_t* out, uint32_t* out_n, uint32_t cap, bool p, uint32_t v, uint32_t* err) {
+  const unsigned m = __ballot_sync(kFull, p);
+  if (m == 0) return;
+  const int ld = __ffs(m) - 1;
+  uint32_t pos = 0;
+  if ((threadIdx.x & 31) == static_cast<uint32_t>(ld)) pos = atomicAdd(out_n, static_cast<uint32_t>(__popc(m)));
+  pos = __shfl_sync(kFull, pos, ld) + __popc(m & lanemask_lt());
+  if (p) {
+    if (pos < cap) out[pos] = v;
+    else atomicCAS(err, DERR_NONE, DERR_WL_OVERFLOW);
+  }
 }
 
-// Relax edge k of a popped vertex whose operator value is `val`
-// (BFS: the level to assign; SSSP: its distance; CC: its label).
+// Relax edge k of a popped vertex whose operator value is `val` (BFS: the level
+// to assign; SSSP: its distance; CC: its label): true when v is to be pushed.
 template <uint32_t OP>
-__device__ __forceinline__ void smem_relax(const uint32_t* col, const uint32_t* w, uint32_t* val_arr,
-                                           uint32_t* stamp, uint32_t k, uint32_t val, uint32_t r, uint32_t* out,
-                                           uint32_t* out_n, uint32_t cap, uint32_t* err) {
-  const uint32_t v = col[k];
-  if (OP == OP_BFS) {
-    if (val_arr[v] == kInf && atomicCAS(val_arr + v, kInf, val) == kInf) smem_push<OP>(out, out_n, cap, v, err);
-    return;
-  }
+__device__ __forceinline__ bool smem_relax(const uint32_t* w, uint32_t* val_arr, uint32_t* stamp, uint32_t k, uint32_t v,
+                                           uint32_t val, uint32_t r) {
+  if (OP == OP_BFS) return val_arr[v] == kInf && atomicCAS(val_arr + v, kInf, val) == kInf;
   const uint32_t nd = OP == OP_SSSP ? val + w[k] : val;
-  if (nd >= val_arr[v]) return;
-  if (nd < atomicMin(val_arr + v, nd) && atomicExch(stamp + v, r) != r) smem_push<OP>(out, out_n, cap, v, err);
+  return nd < val_arr[v] && nd < atomicMin(val_arr + v, nd) && atomicExch(stamp + v, r) != r;
 }
 
 template <uint32_t OP>
 __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
   extern __shared__ __align__(16) uint32_t sh[];
-  __shared__ uint32_t s_n[2];
+  __shared__ uint32_t s_n[3];  // worklist sizes by round mod 3
   __shared__ uint32_t s_err;
   __shared__ unsigned long long s_edges;
   const unsigned long long t_start = p.trace ? globaltimer_ns() : 0ull;
@@ -68,8 +80,7 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
   uint32_t* wl0 = stamp + (OP == OP_BFS ? 0u : n);
   uint32_t* wl1 = wl0 + n;
   if (tid == 0) {
-    s_n[0] = 0;
-    s_n[1] = 0;
+    s_n[0] = s_n[1] = s_n[2] = 0;
     s_err = DERR_NONE;
     s_edges = 0;
   }
@@ -86,67 +97,112 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
   __syncthreads();
   // round-0 worklist: the caller's initial items (CC without them: every vertex)
   const uint32_t init_n = p.init_count ? min(__ldcg(p.init_count), p.init_cap) : n;
-  for (uint32_t i = tid; i < init_n; i += kSmemCta) {
-    const uint32_t s = p.init_items ? __ldcg(p.init_items + i) : i;
-    if (s >= n) {
-      atomicCAS(&s_err, DERR_NONE, DERR_BAD_ITEM);
-      continue;
+  for (uint32_t base = 0; base < init_n; base += kSmemCta) {
+    const uint32_t i = base + tid;
+    bool push = false;
+    uint32_t s = 0;
+    if (i < init_n) {
+      s = p.init_items ? __ldcg(p.init_items + i) : i;
+      // a repeated source or item is pushed once (CC: a mark no round id reaches, rounds stay below n)
+      if (s >= n) atomicCAS(&s_err, DERR_NONE, DERR_BAD_ITEM);
+      else push = OP == OP_CC ? atomicExch(stamp + s, kInitMark) != kInitMark : atomicExch(val + s, 0u) != 0u;
     }
-    if (OP == OP_CC) {
-      // a repeated item is pushed once (a mark no round id reaches: rounds stay below n)
-      if (atomicExch(stamp + s, kInitMark) != kInitMark) smem_push<OP>(wl0, &s_n[0], n, s, &s_err);
-    } else if (atomicExch(val + s, 0u) != 0u) {  // a repeated source is pushed once
-      smem_push<OP>(wl0, &s_n[0], n, s, &s_err);
-    }
+    smem_push(wl0, &s_n[0], n, push, s, &s_err);
   }
   __syncthreads();
   trace_prologue(p.trace, p.trace_cap, t_start, s_n[0]);
+  const uint32_t warp = tid >> 5;
   uint32_t edges = 0, rounds = 0, last_out = 0;
   for (uint32_t r = 0;; ++r) {
     uint32_t* in = (r & 1) ? wl1 : wl0;
     uint32_t* out = (r & 1) ? wl0 : wl1;
-    uint32_t* out_n = &s_n[(r + 1) & 1];
-    const uint32_t in_n = min(s_n[r & 1], n);  // a worklist holds at most n items
-    // every thread has read in_n before the counter is reused two rounds on
-    __syncthreads();
-    if (tid == 0) *out_n = 0;
-    __syncthreads();
-    for (uint32_t base = 0; base < in_n; base += kSmemCta) {
-      const uint32_t i = base + tid;
-      uint32_t b = 0, e = 0, x = 0;
-      if (i < in_n) {
-        const uint32_t u = in[i];
-        b = rp[u];
-        e = rp[u + 1];
-        x = OP == OP_BFS ? r + 1u : val[u];
+    uint32_t* out_n = &s_n[(r + 1) % 3];
+    const uint32_t in_n = min(s_n[r % 3], n);  // a worklist holds at most n items
+    // the counter of round r + 1's pushes: last read at the start of round r - 1, before its barrier
+    if (tid == 0) s_n[(r + 2) % 3] = 0;
+    if (in_n <= kSmemFour) {
+      // Four lanes per item, items dealt across the warps: a short list is one
+      // step of one warp, no search for an edge's owner
+      const uint32_t i = (lane >> 2) * kSmemWarps + warp, sub = lane & 3;
+      if (warp < in_n) {
+        uint32_t b = 0, e = 0, x = 0;
+        if (i < in_n) {
+          const uint32_t u = in[i];
+          b = rp[u];
+          e = rp[u + 1];
+          x = OP == OP_BFS ? r + 1u : val[u];
+        }
+        if (sub == 0) edges += e - b;
+        const bool lng = e - b > 32u;
+        const uint32_t trips = __reduce_max_sync(kFull, lng ? 0u : (e - b + 3u) >> 2);
+        for (uint32_t t = 0; t < trips; ++t) {
+          const uint32_t k = b + 4u * t + sub;
+          const bool mine = !lng && k < e;
+          const uint32_t v = mine ? col[k] : 0u;
+          smem_push(out, out_n, n, mine && smem_relax<OP>(w, val, stamp, k, v, x, r), v, &s_err);
+        }
+        for (unsigned mk = __ballot_sync(kFull, lng && sub == 0); mk; mk &= mk - 1) {
+          const int ld = __ffs(mk) - 1;
+          const uint32_t lb = __shfl_sync(kFull, b, ld), le = __shfl_sync(kFull, e, ld);
+          const uint32_t lx = __shfl_sync(kFull, x, ld);
+          for (uint32_t k0 = lb; k0 < le; k0 += 32) {
+            const uint32_t k = k0 + lane;
+            const uint32_t v = k < le ? col[k] : 0u;
+            smem_push(out, out_n, n, k < le && smem_relax<OP>(w, val, stamp, k, v, lx, r), v, &s_err);
+          }
+        }
       }
-      edges += e - b;
-      // short lists by their own thread, long ones by the whole warp
-      bool lng = e - b > 8u;
-      if (!lng)
-        for (uint32_t k = b; k < e; ++k) smem_relax<OP>(col, w, val, stamp, k, x, r, out, out_n, n, &s_err);
-      for (;;) {
-        const unsigned mk = __ballot_sync(kFull, lng);
-        if (mk == 0) break;
-        const int ld = __ffs(mk) - 1;
-        const uint32_t lb = __shfl_sync(kFull, b, ld), le = __shfl_sync(kFull, e, ld);
-        const uint32_t lx = __shfl_sync(kFull, x, ld);
-        for (uint32_t k = lb + lane; k < le; k += 32) smem_relax<OP>(col, w, val, stamp, k, lx, r, out, out_n, n, &s_err);
-        if (lane == static_cast<uint32_t>(ld)) lng = false;
+    } else {
+      // The warp's items (dealt across the warps) have their edges dealt out to
+      // its lanes, two per lane and step, owners by a shuffle search
+      for (uint32_t base = 0; base < in_n; base += kSmemCta) {
+        const uint32_t i = base + lane * kSmemWarps + warp;
+        uint32_t b = 0, d = 0, x = 0;
+        if (i < in_n) {
+          const uint32_t u = in[i];
+          b = rp[u];
+          d = rp[u + 1] - b;
+          x = OP == OP_BFS ? r + 1u : val[u];
+        }
+        edges += d;
+        const uint32_t incl = warp_incl_scan(d), excl = incl - d;
+        const uint32_t total = __shfl_sync(kFull, incl, 31);
+        for (uint32_t s = 0; s < total; s += 64) {
+          uint32_t k[2], v[2], xx[2];
+          bool mine[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const uint32_t ed = s + 32u * j + lane;
+            mine[j] = ed < total;
+            const uint32_t own = warp_find<uint32_t>(excl, mine[j] ? ed : total - 1u, 32);
+            k[j] = __shfl_sync(kFull, b - excl, own) + ed;
+            xx[j] = __shfl_sync(kFull, x, own);
+            v[j] = mine[j] ? col[k[j]] : 0u;
+          }
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const bool push = mine[j] && smem_relax<OP>(w, val, stamp, k[j], v[j], xx[j], r);
+            smem_push(out, out_n, n, push, v[j], &s_err);
+          }
+        }
       }
     }
-    __syncthreads();
+    // the round's pushes are in; the only barrier of a round, and the error flag with it
+    // (read after it, a thread already in the next round could split the CTA's decision)
+    const int bad = __syncthreads_or(*reinterpret_cast<volatile uint32_t*>(&s_err) != DERR_NONE);
     last_out = min(*out_n, n);
     rounds = r + 1;
     trace_round(p.trace, p.trace_cap, rounds, in_n, last_out);
-    if (last_out == 0 || s_err != DERR_NONE) break;
+    if (last_out == 0 || bad) break;
     if (rounds >= p.max_rounds) {
       if (tid == 0) atomicCAS(&s_err, DERR_NONE, DERR_MAX_ROUNDS);
       break;
     }
   }
   for (uint32_t v = tid; v < n; v += kSmemCta) __stcg(p.state + v, val[v]);
-  atomicAdd(&s_edges, static_cast<unsigned long long>(edges));
+  // summed per warp: a 64-bit shared atomic by each of the 1024 threads took 13 us
+  edges = __reduce_add_sync(kFull, edges);
+  if (lane == 0) atomicAdd(&s_edges, static_cast<unsigned long long>(edges));
   __syncthreads();
   trace_end(p.trace, p.trace_cap, rounds);
   if (tid == 0) {
