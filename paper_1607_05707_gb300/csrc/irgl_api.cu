@@ -226,7 +226,7 @@ irgl_status ensure_workspace(irgl_ctx* ctx, uint32_t n, bool need_stamp, bool ne
 }
 
 int occupancy(irgl_ctx* ctx, int kind, uint32_t op, uint32_t cta, int red) {
-  const int key = ((kind * 8 + static_cast<int>(op)) * 5 + (static_cast<int>(cta) >> 8)) * 3 + red;
+  const int key = ((kind * 16 + static_cast<int>(op)) * 5 + (static_cast<int>(cta) >> 8)) * 3 + red;
   auto it = ctx->occ.find(key);
   if (it != ctx->occ.end()) return it->second;
   int nb = 0;
@@ -820,7 +820,8 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   // a vertex can be pushed once per sub-round: worklists of n * (sub-rounds + 1)
   s = ensure_workspace(ctx, g->n, k != IRGL_BFS, far, vis, packed, use_local ? sub_rounds + 1u : 1u);
   if (s != IRGL_OK) return s;
-  const uint32_t op = (use_local && k == IRGL_BFS) ? OP_BFSR : op_of(k);
+  const uint32_t op = use_local ? (k == IRGL_BFS ? OP_BFSR : OP_SSSPL)
+                      : far ? (k == IRGL_SSSP ? OP_SSSPF : OP_CCF) : op_of(k);
   if (k == IRGL_CC_JUMP) t.cta_size = kUfCta;  // its vertex blocks fill an SM's shared memory: one CTA each
   if (k == IRGL_CC_JUMP && mode != IRGL_PERSISTENT)
     return fail(IRGL_ERR_UNSUPPORTED, "pointer-jumping CC runs only as a persistent Iterate");

@@ -378,7 +378,7 @@ irgl_status irgl_batch_prepare(irgl_batch* b, const irgl_tuning* tin, int use_cu
   }
   // persistent grid
   int nb = 0;
-  e = occupancy_batch(t.cta_size, &nb);
+  e = occupancy_batch(t.cta_size, nf, b->ds != nullptr && ((t.flags >> 8) & 15u) != 0, &nb);
   if (e != cudaSuccess || nb <= 0) {
     batch_free_device(b);
     return fail(IRGL_ERR_CUDA, "batched kernel cannot be made resident");

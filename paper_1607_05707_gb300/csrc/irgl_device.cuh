@@ -36,17 +36,27 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // OP_BFSR: BFS levels by label-correcting relaxation (SSSP with unit weights:
 // a popped vertex's current level + 1), the form the CTA-local sub-rounds need,
 // since a vertex can be reached there before its level is final.
-enum : uint32_t { OP_BFS = 0, OP_SSSP = 1, OP_CC = 2, OP_RUNTIME = 3, OP_CCJ = 4, OP_BFSR = 5 };
+// OP_SSSPF, OP_CCF: SSSP and min-label CC with the near-far schedule, kernels of
+// their own: its lists and limits kept in registers beside the plain rounds' code
+// made the plain SSSP kernel spill (112 bytes of spill loads, 20 without). OP_SSSPL: launch table entry of the
+// SSSP kernel with CTA-local sub-rounds (LOCAL below).
+enum : uint32_t { OP_BFS = 0, OP_SSSP = 1, OP_CC = 2, OP_RUNTIME = 3, OP_CCJ = 4, OP_BFSR = 5, OP_SSSPL = 6, OP_SSSPF = 7,
+                  OP_CCF = 8 };
 
-// Operators whose values can be scheduled near-far (smallest first): SSSP
-// distances and min-label CC labels.
+// The operator an id stands for.
+__host__ __device__ constexpr uint32_t base_op(uint32_t op) {
+  return op == OP_SSSPF || op == OP_SSSPL ? static_cast<uint32_t>(OP_SSSP) : op == OP_CCF ? static_cast<uint32_t>(OP_CC) : op;
+}
+
+// Operators whose values are scheduled near-far (smallest first): SSSP distances
+// and min-label CC labels.
 template <uint32_t OP>
-constexpr bool kNearFarOp = OP == OP_SSSP || OP == OP_CC;
+constexpr bool kNearFarOp = OP == OP_SSSPF || OP == OP_CCF;
 
 // Operators that can keep (value, round id) in one 64-bit word per vertex:
 // single-graph SSSP, and every query of the batched kernel.
 template <uint32_t OP>
-constexpr bool kPackedOp = OP == OP_SSSP || OP == OP_RUNTIME || OP == OP_BFSR;
+constexpr bool kPackedOp = base_op(OP) == OP_SSSP || OP == OP_RUNTIME || OP == OP_BFSR;
 enum : int { RED_NONE = 0, RED_ANY = 1, RED_ALL = 2 };
 // Device error codes (first one wins).
 enum : uint32_t {
@@ -386,13 +396,24 @@ struct Smem {
   uint8_t pushed[CTA];                      // ReduceAndReturn All: item pushed something
 };
 
-template <int CTA>
+// Far items of a batched launch staged per CTA: the far list is appended with one
+// atomic per flush instead of one per pushing warp on its single counter. With the
+// sparse round's even deal of the far items and limits that rise in the round that
+// drained a query, 91 SSSP queries on grids went from 332 rounds and 36 ms to 177
+// rounds and 12.5 ms.
+constexpr uint32_t kFarStage = 1024;
+
+template <int CTA, bool NF>
 struct BatchSmem {
   Smem<CTA> core;
   uint32_t sbases[kMaxBatchQueries];
   uint32_t qbits[kMaxBatchQueries / 32];  // queries (by slot) this CTA pushed for in the current round
-  uint32_t qfar[kMaxBatchQueries / 32];   // queries (by slot) this CTA kept on the far list
-  uint32_t lim[kMaxBatchQueries];         // near-far: this round's limit of each query (by id)
+  uint32_t qfar[kMaxBatchQueries / 32];   // queries (by slot) active otherwise: items kept on the far
+                                          // list, pushes already expanded by the sub-rounds
+  uint32_t lim[NF ? kMaxBatchQueries : 1];  // near-far: this round's limit of each query (by id)
+  uint32_t far_stage[NF ? kFarStage : 1u];  // far items on their way to the far list
+  uint32_t far_n;
+  uint32_t dmin[NF ? 1 : kMaxBatchQueries];  // by slot: the smallest SSSP distance this CTA pushed this round
 };
 
 // ----------------------------------------------------------------------------- cooperative-conversion push
@@ -558,9 +579,9 @@ struct SingleView {
   uint32_t* stamp;
   uint32_t n;
   static constexpr bool kBatched = false;
-  static constexpr const uint32_t* lim = nullptr;
+  static constexpr bool kNear = false;
   __device__ __forceinline__ uint32_t nverts(uint32_t) const { return n; }
-  __device__ __forceinline__ uint32_t op(uint32_t) const { return OP; }
+  __device__ __forceinline__ uint32_t op(uint32_t) const { return base_op(OP); }
   __device__ __forceinline__ const uint32_t* rowp(uint32_t) const { return row_ptr; }
   __device__ __forceinline__ const uint32_t* colp(uint32_t) const { return col; }
   __device__ __forceinline__ const int32_t* wp(uint32_t) const { return w; }
@@ -570,8 +591,11 @@ struct SingleView {
   __device__ __forceinline__ uint32_t slot(uint32_t) const { return 0u; }
 };
 
-// Many queries over many graphs; op taken per query at run time.
+// Many queries over many graphs; op taken per query at run time. NF: near-far
+// (per-query limits) may be on.
+template <bool NF>
 struct BatchView {
+  static constexpr bool kNear = NF;
   const QDesc* __restrict__ desc;
   const uint32_t* sbases;  // shared-memory copy
   uint32_t nq;
@@ -581,6 +605,9 @@ struct BatchView {
   uint32_t* qfar;   // shared-memory bitmap of queries that kept far items this round
   const uint32_t* lim;  // near-far: per-query limits (shared memory), or nullptr
   uint32_t* far_stamp;
+  uint32_t* far_stage;  // near-far: kFarStage entries of shared memory and their count
+  uint32_t* far_n;
+  uint32_t* dmin;       // deferred expansion: by slot, the smallest distance this CTA pushed this round (shared memory)
   static constexpr bool kBatched = true;
   __device__ __forceinline__ uint32_t op(uint32_t q) const { return __ldg(&desc[q].op); }
   __device__ __forceinline__ const uint32_t* rowp(uint32_t q) const {
@@ -611,10 +638,19 @@ struct BatchView {
     const uint32_t slot = __ldg(&desc[q].slot);
     atomicOr(&qbits[slot >> 5], 1u << (slot & 31u));
   }
-  // near-far: the query holds far items (still active, but no out-worklist push)
-  __device__ __forceinline__ void mark_far(uint32_t q) const {
-    const uint32_t slot = __ldg(&desc[q].slot);
-    atomicOr(&qfar[slot >> 5], 1u << (slot & 31u));
+  // deferred expansion: a distance the query pushed this round; the CTA's smallest
+  // per query go to the round's global words once, before the barrier (combining the
+  // lanes of every strip with match and reduce for a global atomic instead cost the
+  // 256-instance batch 6.4 ms against 5.5)
+  __device__ __forceinline__ void note(uint32_t q, uint32_t nd) const { atomicMin(dmin + __ldg(&desc[q].slot), nd); }
+  // the query is still active, but nothing of it went to the out-worklist (far
+  // items kept, or pushes that the sub-rounds expand themselves). Most find their
+  // bit set: a read, then an atomic only if it is not (mark() stays without the
+  // read: nothing waits for its atomic, and the read cost the R-MAT batch 4 %)
+  __device__ __forceinline__ void mark_active(uint32_t q) const {
+    const uint32_t slot = __ldg(&desc[q].slot), bit = 1u << (slot & 31u);
+    uint32_t* const w = qfar + (slot >> 5);
+    if ((*reinterpret_cast<volatile uint32_t*>(w) & bit) == 0u) atomicOr(w, bit);
   }
 };
 
@@ -627,7 +663,7 @@ struct BatchView {
 template <uint32_t OP>
 __device__ __forceinline__ bool relax(uint32_t op_rt, uint32_t* state, uint32_t* stamp, uint32_t v, uint32_t val,
                                       int32_t wt, uint32_t ep) {
-  const uint32_t op = OP == OP_RUNTIME ? op_rt : OP;
+  const uint32_t op = OP == OP_RUNTIME ? op_rt : base_op(OP);
   if (op == OP_BFS) {
     if (__ldcg(state + v) != kInf) return false;
     return atomicCAS(state + v, kInf, val) == kInf;
@@ -644,7 +680,7 @@ __device__ __forceinline__ bool relax(uint32_t op_rt, uint32_t* state, uint32_t*
 template <uint32_t OP>
 __device__ __forceinline__ bool decide(uint32_t op_rt, uint32_t* state, uint32_t* stamp, uint32_t v, uint32_t val,
                                        int32_t wt, uint32_t cur, uint32_t ep) {
-  const uint32_t op = OP == OP_RUNTIME ? op_rt : OP;
+  const uint32_t op = OP == OP_RUNTIME ? op_rt : base_op(OP);
   if (op == OP_BFS) {
     if (cur != kInf) return false;
     return atomicCAS(state + v, kInf, val) == kInf;
@@ -658,7 +694,7 @@ __device__ __forceinline__ bool decide(uint32_t op_rt, uint32_t* state, uint32_t
 
 template <uint32_t OP>
 __device__ __forceinline__ bool needs_w(uint32_t op_rt) {
-  return (OP == OP_RUNTIME ? op_rt : OP) == OP_SSSP;
+  return (OP == OP_RUNTIME ? op_rt : base_op(OP)) == OP_SSSP;
 }
 
 // ----------------------------------------------------------------------------- one tile of items
@@ -706,17 +742,6 @@ struct RoundCtx {
   uint32_t* bdmin_next = nullptr;
   uint32_t defer_delta = 0;
 };
-
-// Batched deferred expansion: lanes that pushed SSSP distances for the same
-// query slot combine their smallest into one atomic on that slot's word of
-// the round's buffer (stored complemented, so 0 means nothing pushed). Every
-// lane of the warp calls it; mn = kInf: nothing to note.
-__device__ __forceinline__ void note_pushes(uint32_t* next, uint32_t slot, uint32_t mn) {
-  const uint32_t key = mn != kInf ? slot : 0xFFFFFFFFu;
-  const unsigned grp = __match_any_sync(kFull, key);
-  const uint32_t gm = __reduce_min_sync(grp, mn);
-  if (key != 0xFFFFFFFFu && (threadIdx.x & 31u) == static_cast<uint32_t>(__ffs(grp) - 1)) atomicMax(next + slot, ~gm);
-}
 
 // The destination's current value as the operator reads it. BFS with the
 // visited bitmap: the bit is read through L1 (a 128 KB bitmap of 2^20 vertices
@@ -807,25 +832,25 @@ __device__ __forceinline__ uint32_t decide_route(uint32_t op_rt, uint32_t* state
     // one 64-bit atomicMin lowers the value and stamps the round: v is
     // pushed by the thread that lowers it first in this round (a far
     // improvement stamps 0: see decide_n). BFS levels are lowered from INF.
-    const uint32_t o = OP == OP_RUNTIME ? op_rt : OP;
+    const uint32_t o = OP == OP_RUNTIME ? op_rt : base_op(OP);
     const uint32_t nd = o == OP_SSSP ? val + static_cast<uint32_t>(wt) : (o == OP_BFSR ? val + 1u : val);
     // batched BFS under CTA-local sub-rounds is label-correcting (as in decide_n)
     const bool first_only = o == OP_BFS && !(OP == OP_RUNTIME && rc.local_rounds != 0);
     if (first_only ? cur != kInf : nd >= cur) return 0u;
-    const bool far = OP == OP_SSSP && rc.limit != kInf && nd >= rc.limit;
+    const bool far = kNearFarOp<OP> && rc.limit != kInf && nd >= rc.limit;
     const unsigned long long old =
         atomicMin(rc.ds + sb + v, (static_cast<unsigned long long>(nd) << 32) | (far ? 0u : rc.dsr));
     if (nd >= static_cast<uint32_t>(old >> 32)) return 0u;
     if (!far) {
       const bool push = static_cast<uint32_t>(old) != rc.dsr;
-      if (OP == OP_SSSP && push && rc.pmin != nullptr) atomicMin(rc.pmin, nd);
+      if (base_op(OP) == OP_SSSP && push && rc.pmin != nullptr) atomicMin(rc.pmin, nd);
       return push ? 1u : 0u;
     }
     nd_out = nd;
     return atomicExch(rc.far_stamp + v, rc.phase) != rc.phase ? 2u : 0u;
   }
   if (!kNearFarOp<OP> || rc.limit == kInf) return decide<OP>(op_rt, state, stamp, v, val, wt, cur, rc.ep) ? 1u : 0u;
-  const uint32_t nd = OP == OP_SSSP ? val + static_cast<uint32_t>(wt) : val;
+  const uint32_t nd = base_op(OP) == OP_SSSP ? val + static_cast<uint32_t>(wt) : val;
   if (nd >= cur) return 0u;
   const uint32_t old = atomicMin(state + v, nd);
   if (nd >= old) return 0u;
@@ -858,7 +883,7 @@ __device__ __forceinline__ void decide_n(const RoundCtx& rc, uint32_t* state, ui
   bool t[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const uint32_t o = OP == OP_RUNTIME ? op[k] : OP;
+    const uint32_t o = OP == OP_RUNTIME ? op[k] : base_op(OP);
     nd[k] = o == OP_SSSP ? val[k] + static_cast<uint32_t>(wt[k]) : (o == OP_BFSR ? val[k] + 1u : val[k]);
     // BFS takes unvisited vertices only, except batched BFS under CTA-local
     // sub-rounds, where a vertex can be reached before its level is final
@@ -880,7 +905,7 @@ __device__ __forceinline__ void decide_n(const RoundCtx& rc, uint32_t* state, ui
 #pragma unroll
     for (int k = 0; k < N; ++k)
       r[k] = (t[k] && nd[k] < static_cast<uint32_t>(old[k] >> 32) && static_cast<uint32_t>(old[k]) != rc.dsr) ? 1u : 0u;
-    if (OP == OP_SSSP && rc.pmin != nullptr) {
+    if (base_op(OP) == OP_SSSP && rc.pmin != nullptr) {
       uint32_t mn = kInf;
 #pragma unroll
       for (int k = 0; k < N; ++k) mn = r[k] ? min(mn, nd[k]) : mn;
@@ -888,7 +913,7 @@ __device__ __forceinline__ void decide_n(const RoundCtx& rc, uint32_t* state, ui
     }
     return;
   }
-  if (OP == OP_SSSP && rc.ds != nullptr) {
+  if (OP == OP_SSSPF && rc.ds != nullptr) {
     // A far improvement writes round id 0: the vertex is not on this round's
     // out-worklist (its value was >= the limit, so no near push happened this
     // round), and a later near improvement in the round must still push it.
@@ -914,7 +939,7 @@ __device__ __forceinline__ void decide_n(const RoundCtx& rc, uint32_t* state, ui
   uint32_t old[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const uint32_t o = OP == OP_RUNTIME ? op[k] : OP;
+    const uint32_t o = OP == OP_RUNTIME ? op[k] : base_op(OP);
     uint32_t* const s = state + sb[k] + v[k];
     old[k] = 0u;
     if (t[k]) old[k] = o == OP_BFS ? atomicCAS(s, kInf, nd[k]) : atomicMin(s, nd[k]);
@@ -923,7 +948,7 @@ __device__ __forceinline__ void decide_n(const RoundCtx& rc, uint32_t* state, ui
   uint32_t ex[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const uint32_t o = OP == OP_RUNTIME ? op[k] : OP;
+    const uint32_t o = OP == OP_RUNTIME ? op[k] : base_op(OP);
     imp[k] = t[k] && (o == OP_BFS ? old[k] == kInf : nd[k] < old[k]);
     ex[k] = far[k] ? ~rc.phase : ~rc.ep;
     if (imp[k] && o != OP_BFS)
@@ -931,7 +956,7 @@ __device__ __forceinline__ void decide_n(const RoundCtx& rc, uint32_t* state, ui
   }
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const uint32_t o = OP == OP_RUNTIME ? op[k] : OP;
+    const uint32_t o = OP == OP_RUNTIME ? op[k] : base_op(OP);
     r[k] = (imp[k] && (o == OP_BFS || ex[k] != (far[k] ? rc.phase : rc.ep))) ? (far[k] ? 2u : 1u) : 0u;
     if (OP == OP_BFS && r[k] != 0u) {
       if (rc.vis) atomicOr(rc.vis + (v[k] >> 5), 1u << (v[k] & 31u));
@@ -1032,7 +1057,7 @@ __device__ __forceinline__ bool group_edges(const V& g, Smem<CTA>& sm, const Rou
     push4<CTA>(sm, rc.out, fn, sb + c.x, sb + c.y, sb + c.z, sb + c.w);
     if (kNearFarOp<OP>) push_far4<CTA>(sm, rc.far_out, ff, sb + c.x, sb + c.y, sb + c.z, sb + c.w, dmin);
     if constexpr (V::kBatched) {
-      if (rc.bdmin_next != nullptr) note_pushes(rc.bdmin_next, g.slot(q), op == OP_SSSP ? pmn : kInf);
+      if (rc.bdmin_next != nullptr && op == OP_SSSP && pmn != kInf) g.note(q, pmn);
     }
     any |= (fn | ff) != 0;
     if (GROUP == CTA) {
@@ -1055,9 +1080,37 @@ __device__ __forceinline__ void push_far_item(const V& g, Smem<CTA>& sm, const R
   bool f = false;
   if (want) {
     f = atomicExch(g.far_stamp + item, rc.ep) != rc.ep;
-    g.mark_far(q);
+    g.mark_active(q);
   }
-  push_far4<CTA>(sm, rc.far_out, f ? 1u : 0u, item, 0u, 0u, 0u, kInf);
+  const unsigned m = __ballot_sync(kFull, f);
+  if (m == 0) return;
+  const int ld = __ffs(m) - 1;
+  const uint32_t cnt = __popc(m);
+  uint32_t base = 0;
+  if ((threadIdx.x & 31) == static_cast<uint32_t>(ld)) base = atomicAdd(g.far_n, cnt);
+  base = __shfl_sync(kFull, base, ld);
+  const uint32_t pos = base + __popc(m & lanemask_lt());
+  if (f && pos < kFarStage) g.far_stage[pos] = item;
+  if (base + cnt > kFarStage)  // the stage is full: straight to the list
+    push_far4<CTA>(sm, rc.far_out, f && pos >= kFarStage ? 1u : 0u, item, 0u, 0u, 0u, kInf);
+}
+
+// Append the staged far items (more than `above` of them) to the far list. Every
+// thread of the CTA, at a CTA-uniform point.
+template <int CTA, class V>
+__device__ __forceinline__ void flush_far(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t above) {
+  if (!__syncthreads_or(*g.far_n > above)) return;
+  const uint32_t n = min(*g.far_n, kFarStage);
+  if (threadIdx.x == 0) sm.gbase = atomicAdd(rc.far_out.tail, n);
+  __syncthreads();
+  const uint32_t gb = sm.gbase;
+  for (uint32_t i = threadIdx.x; i < n; i += CTA) {
+    if (gb + i < rc.far_out.cap) __stcg(rc.far_out.items + gb + i, g.far_stage[i]);
+    else set_err(rc.far_out.err, DERR_WL_OVERFLOW);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *g.far_n = 0;
+  __syncthreads();
 }
 
 // Put the round id `dsr` into a packed (value, round id) word whose value it
@@ -1098,10 +1151,11 @@ __device__ __forceinline__ void far_sweep(const V& g, Smem<CTA>& sm, const Round
     }
     push1<CTA>(sm, rc.out, near, item);
     push_far_item<CTA>(g, sm, rc, keep, item, q);
+    flush_far<CTA>(g, sm, rc, kFarStage / 2);
   }
 }
 
-template <uint32_t OP, int CTA, int RED, class V>
+template <uint32_t OP, int CTA, int RED, bool LOCAL, class V>
 __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t idx,
                                              uint32_t& edges, uint32_t& any_true, uint32_t& any_false) {
   const uint32_t tid = threadIdx.x;
@@ -1111,7 +1165,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
   uint32_t q = 0, beg = 0, end = 0, val = 0, item = 0;
   unsigned long long pw = 0;  // the popped packed word (single-query SSSP)
   if (valid) {
-    item = rc.local_items ? rc.local_items[idx] : (rc.in_items ? __ldcg(rc.in_items + idx) : idx);
+    item = LOCAL && rc.local_items ? rc.local_items[idx] : (rc.in_items ? __ldcg(rc.in_items + idx) : idx);
     uint32_t u;
     g.decode(item, q, u);
     uint32_t dval = 0;
@@ -1139,7 +1193,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
       beg = __ldg(rp + u);
       end = __ldg(rp + u + 1);
       const uint32_t op = g.op(q);
-      if (kPackedOp<OP> && rc.ds != nullptr && rc.local_items != nullptr)
+      if (LOCAL && kPackedOp<OP> && rc.ds != nullptr && rc.local_items != nullptr)
         // a CTA-local pop: take the value and clear the round stamp in one
         // atomic, so an improvement that lands after this read (from any CTA,
         // in any sub-round) pushes the vertex again instead of counting on a
@@ -1156,7 +1210,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
       else val = __ldcg(g.state + item);
     }
   }
-  if constexpr (!V::kBatched && OP == OP_SSSP) {
+  if constexpr (!V::kBatched && OP == OP_SSSP && !LOCAL) {
     // Deferred expansion of long lists: a vertex of degree >= defer_deg whose
     // distance is above defer_lim (the smallest distance pushed for this round
     // plus a margin) is likely to be lowered again before it is final, and each
@@ -1165,7 +1219,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
     // its distance counted in the round's smallest, so the smallest item of a
     // round is never deferred and every vertex is expanded in the end.
     bool again = false;
-    if (valid && rc.defer_lim != kInf && !rc.dense && rc.local_items == nullptr && end - beg >= rc.defer_deg &&
+    if (valid && rc.defer_lim != kInf && !rc.dense && end - beg >= rc.defer_deg &&
         val > rc.defer_lim) {
       again = stamp_pending(rc.ds + item, pw, rc.dsr);
       if (again) atomicMin(rc.pmin, val);
@@ -1174,18 +1228,18 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
     }
     if (rc.defer_lim != kInf) push1<CTA>(sm, rc.out, again, item);
   }
-  if constexpr (V::kBatched) {
+  if constexpr (V::kBatched && !LOCAL) {
     // the same for SSSP queries of a batch, each against its own smallest
     // pushed distance of the last round (its slot's word; 0: none noted)
     bool again = false;
-    if (rc.bdmin_cur != nullptr && valid && rc.local_items == nullptr && end - beg >= rc.defer_deg &&
+    if (rc.bdmin_cur != nullptr && valid && end - beg >= rc.defer_deg &&
         g.op(q) == OP_SSSP) {
       const uint32_t sl = g.slot(q);
       const uint32_t pm = __ldcg(rc.bdmin_cur + sl);
       if (pm != 0u && static_cast<unsigned long long>(val) > static_cast<unsigned long long>(~pm) + rc.defer_delta) {
         again = stamp_pending(rc.ds + item, pw, rc.dsr);
         if (again) {
-          atomicMax(rc.bdmin_next + sl, ~val);
+          g.note(q, val);
           g.mark(q, rc.ep);
         }
         valid = false;
@@ -1194,7 +1248,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
     }
     if (rc.bdmin_cur != nullptr) push1<CTA>(sm, rc.out, again, item);
   }
-  if constexpr (V::kBatched) {
+  if constexpr (V::kNear) {
     if (g.lim != nullptr) {
       // near-far: an SSSP item at or above its query's limit is not expanded
       // now; it waits on the far list (once per round) until the limit passes it
@@ -1385,7 +1439,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
       if (rc.bdmin_next != nullptr) {
 #pragma unroll
         for (uint32_t k = 0; k < E; ++k)
-          note_pushes(rc.bdmin_next, g.slot(oqs[k]), (rr[k] == 1u && op[k] == OP_SSSP) ? ndv[k] : kInf);
+          if (rr[k] == 1u && op[k] == OP_SSSP) g.note(oqs[k], ndv[k]);
       }
     }
     push4<CTA>(sm, rc.out, f, sb[0] + v[0], sb[1] + v[1], sb[2] + v[2], sb[3] + v[3]);
@@ -1395,7 +1449,7 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
 
   if (RED == RED_ANY) any_true |= pushed ? 1u : 0u;
   // a sub-round reads its items from the stage: no flush may move them under it
-  const bool full = __syncthreads_or(rc.local_items == nullptr &&
+  const bool full = __syncthreads_or((!LOCAL || rc.local_items == nullptr) &&
                                      sm.stage_n >= static_cast<uint32_t>(Smem<CTA>::kStage / 2));
   if (RED == RED_ALL) {
     if (valid && !sm.pushed[tid]) any_false = 1u;
@@ -1404,16 +1458,268 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
   if (full) flush_stage<CTA>(sm, rc.out);
 }
 
+// ----------------------------------------------------------------------------- sparse round with sub-rounds
+
+// A round of a launch with CTA-local sub-rounds whose frontier is below one tile
+// per CTA: the CTA's share of the in-worklist (items b, b + grid, ...) and, after
+// it, what its own pushes discover, sub-round by sub-round, with CTA barriers
+// only. Same pops, stamps and pushes as process_tile under sub-rounds (a global
+// pop reads its word, a local pop clears the stamp in the read; see round_body). A
+// batched query is marked as holding out-worklist items only for what is left when
+// the round ends: with near-far its limit then rises in the round that drained it.
+//
+// What bounds it: a chain of dependent reads per sub-round, not bandwidth (4096^2
+// mesh BFS: a few thousand items over 1216 CTAs). Through process_tile the chain
+// was row offsets -> column -> neighbour's word -> atomic, with a shuffle scan and
+// a search per edge between them: 3.3 us a sub-round. Here an entry carries its
+// row offsets (read beside the atomicMin that discovers it), a list is dealt to
+// four lanes without a search, and the atomicMin is issued without reading the
+// word first: two dependent reads are left, (own word | columns) -> (atomicMin |
+// the neighbour's row offsets). 4096^2 mesh BFS, 382 rounds of 16 sub-rounds: 54 -> 32 us
+// a round, 16.7 -> 9.9 ms a call; with a read before the atomicMin 11.2 ms.
+//
+// Entries {item, first edge, end (, query)} live in two halves of the stage that
+// alternate; pushes that find a half full go straight to the out-worklist. Lists
+// of at least the split threshold go to the grid-wide big list, as in process_tile.
+template <int CTA, class V>
+struct LocalBuf {
+  static constexpr uint32_t kFields = V::kBatched ? 4 : 3;
+  static constexpr uint32_t kCap = (Smem<CTA>::kStage / (2 * kFields)) & ~31u;  // entries per half
+  static_assert(kCap >= static_cast<uint32_t>(CTA), "room for a tile of the in-worklist");
+};
+
+// Warp-aggregated push of one optional entry per lane to a half of the stage.
+template <int CTA, class V>
+__device__ __forceinline__ void push_local(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t* half, uint32_t* count,
+                                           bool p, uint32_t item, uint32_t beg, uint32_t end, uint32_t q) {
+  constexpr uint32_t C = LocalBuf<CTA, V>::kCap;
+  const unsigned m = __ballot_sync(kFull, p);
+  if (m == 0) return;
+  const int ld = __ffs(m) - 1;
+  const uint32_t cnt = __popc(m);
+  uint32_t base = 0;
+  if ((threadIdx.x & 31) == static_cast<uint32_t>(ld)) base = atomicAdd(count, cnt);
+  base = __shfl_sync(kFull, base, ld);
+  const uint32_t pos = base + __popc(m & lanemask_lt());
+  const bool fits = pos < C;
+  if (p && fits) {
+    half[pos] = item;
+    half[C + pos] = beg;
+    half[2 * C + pos] = end;
+    if (V::kBatched) half[3 * C + pos] = q;
+  }
+  if (base + cnt > C) {
+    if (V::kBatched && p && !fits) g.mark(q, rc.ep);
+    push_global_warp(rc.out, &sm.round_pushes, p && !fits ? 1u : 0u, item, 0u, 0u, 0u);
+  }
+}
+
+template <uint32_t OP, int CTA, class V>
+__device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t& edges) {
+  constexpr uint32_t C = LocalBuf<CTA, V>::kCap;
+  constexpr uint32_t W = CTA / 32;
+  __shared__ uint32_t l_n[3];  // entries by sub-round mod 3
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
+  uint32_t* const half0 = sm.stage;
+  uint32_t* const half1 = sm.stage + LocalBuf<CTA, V>::kFields * C;
+  const uint32_t m = rc.in_n > blockIdx.x ? (rc.in_n - blockIdx.x - 1u) / gridDim.x + 1u : 0u;  // <= CTA
+  if (tid < 3) l_n[tid] = tid == 0 ? m : 0u;
+  __syncthreads();
+  if (tid < m) {
+    const uint32_t idx = blockIdx.x + tid * gridDim.x;
+    uint32_t item = rc.in_items ? __ldcg(rc.in_items + idx) : idx;
+    uint32_t q, u, beg = 0, end = 0;
+    g.decode(item, q, u);
+    if (u < g.nverts(q)) {
+      beg = __ldg(g.rowp(q) + u);
+      end = __ldg(g.rowp(q) + u + 1);
+    } else {  // a caller-pushed item outside the graph: report and skip it
+      set_err(rc.out.err, DERR_BAD_ITEM);
+      item = 0;
+    }
+    half0[tid] = item;
+    half0[C + tid] = beg;
+    half0[2 * C + tid] = end;
+    if (V::kBatched) half0[3 * C + tid] = q;
+  }
+  if constexpr (V::kNear) {
+    // near-far: far items whose query's limit has passed them join this round (as in far_sweep)
+    if (g.lim != nullptr) {
+      // dealt across the CTAs item by item: a query's far items are neighbours on the
+      // list, and the CTAs that release them expand them for the rest of the round
+      // (in blocks of CTA items a few SMs did five times the average's work)
+      const unsigned long long all = static_cast<unsigned long long>(gridDim.x) * CTA;
+      for (unsigned long long base = 0; base < rc.far_in_n; base += all) {
+        const unsigned long long i = base + static_cast<unsigned long long>(tid) * gridDim.x + blockIdx.x;
+        bool near = false, keep = false;
+        uint32_t item = 0, q = 0, beg = 0, end = 0;
+        if (i < rc.far_in_n) {
+          item = __ldcg(rc.far_in + i);
+          uint32_t u;
+          g.decode(item, q, u);
+          const unsigned long long w = __ldcg(rc.ds + item);
+          if (static_cast<uint32_t>(w >> 32) < g.lim[q]) {
+            near = stamp_pending(rc.ds + item, w, rc.dsr);
+            if (near) {
+              g.mark_active(q);
+              beg = __ldg(g.rowp(q) + u);
+              end = __ldg(g.rowp(q) + u + 1);
+            }
+          } else {
+            keep = true;
+          }
+        }
+        push_local<CTA>(g, sm, rc, half0, &l_n[0], near, item, beg, end, q);
+        push_far_item<CTA>(g, sm, rc, keep, item, q);
+        flush_far<CTA>(g, sm, rc, kFarStage / 2);
+      }
+    }
+  }
+  __syncthreads();
+  const uint32_t split = min(rc.tn.warp_thresh, rc.tn.cta_thresh);  // as a frontier below one tile per CTA splits
+  uint32_t j = 0;
+  for (; j <= rc.local_rounds; ++j) {
+    const uint32_t n = min(l_n[j % 3], C);
+    if (n == 0) break;
+    const uint32_t* const cur = (j & 1) ? half1 : half0;
+    uint32_t* const nxt = (j & 1) ? half0 : half1;
+    uint32_t* const nxt_n = &l_n[(j + 1) % 3];
+    if (tid == 0) l_n[(j + 2) % 3] = 0;  // last read before the barrier that ended sub-round j - 1
+    const uint32_t dsr = rc.dsr + j;
+    for (uint32_t base = warp; base < n; base += CTA / 4) {  // warp-uniform: items base, base + W, ..., base + 7 W
+      const uint32_t idx = base + (lane >> 2) * W;
+      const bool valid = idx < n;
+      const uint32_t item = valid ? cur[idx] : 0u;
+      uint32_t beg = valid ? cur[C + idx] : 0u, end = valid ? cur[2 * C + idx] : 0u;
+      const uint32_t q = V::kBatched && valid ? cur[3 * C + idx] : 0u;
+      const uint32_t op = valid ? g.op(q) : static_cast<uint32_t>(OP_BFS);
+      // the item's word and its first columns in flight together
+      unsigned long long word = 0;
+      if (valid && sub == 0) {
+        if (j == 0 && idx < m) word = __ldcg(rc.ds + item);
+        else word = atomicAnd(rc.ds + item, 0xFFFFFFFF00000000ull);
+      }
+      const uint32_t* const col = g.colp(q);
+      const int32_t* const w = g.wp(q);
+      const uint32_t* const rowp = g.rowp(q);
+      const uint32_t sb = g.sbase(q);
+      const bool nw = valid && needs_w<OP>(op);
+      uint32_t c = beg + sub < end ? __ldg(col + beg + sub) : 0u;
+      uint32_t add = (OP == OP_BFSR) ? 1u : (nw && beg + sub < end ? static_cast<uint32_t>(__ldg(w + beg + sub)) : 0u);
+      // the value the out-edges start from (a batched BFS item: the level they assign)
+      const uint32_t val = __shfl_sync(kFull, static_cast<uint32_t>(word >> 32), lane & ~3u) +
+                           (OP == OP_RUNTIME && op == OP_BFS ? 1u : 0u);
+      if constexpr (V::kNear) {
+        if (g.lim != nullptr) {
+          const bool defer = valid && op == OP_SSSP && val >= g.lim[q];
+          push_far_item<CTA>(g, sm, rc, defer && sub == 0, item, q);
+          if (defer) end = beg;
+        }
+      }
+      const uint32_t deg = end - beg;
+      if (sub == 0) edges += deg;
+      if (__any_sync(kFull, deg >= split && rc.big.cap != 0)) {
+        bool listed = false;
+        if (sub == 0 && deg >= split) {
+          const unsigned long long at = atomicAdd(rc.big_ctr, (1ull << 40) | deg);
+          const uint32_t slot = static_cast<uint32_t>(at >> 40);
+          sm.big_appended = 1;
+          if (slot < rc.big.cap) {
+            rc.big.e[slot] = make_uint4(beg, end, val, q);
+            rc.big.off[slot] = at & kBigEdgeMask;
+            listed = true;
+          }
+        }
+        if (__shfl_sync(kFull, listed ? 1u : 0u, lane & ~3u)) end = beg;
+      }
+      // four lanes per list; lists of more than 32 edges (big list off or full) by the warp
+      const bool lng = end - beg > 32u;
+      const uint32_t trips = __reduce_max_sync(kFull, lng ? 0u : (end - beg + 3u) >> 2);
+      for (uint32_t t = 0; t < trips; ++t) {
+        const uint32_t k = beg + 4u * t + sub;
+        const bool mine = !lng && k < end;
+        unsigned long long old = 0;
+        uint32_t nb = 0, ne = 0;
+        const uint32_t nd = val + add, v = c;
+        if (mine) {
+          old = atomicMin(rc.ds + sb + v, (static_cast<unsigned long long>(nd) << 32) | dsr);
+          nb = __ldg(rowp + v);
+          ne = __ldg(rowp + v + 1);
+        }
+        if (k + 4u < end && !lng) {
+          c = __ldg(col + k + 4u);
+          if (nw) add = static_cast<uint32_t>(__ldg(w + k + 4u));
+        }
+        const bool push = mine && nd < static_cast<uint32_t>(old >> 32) && static_cast<uint32_t>(old) != dsr;
+        if constexpr (V::kBatched) {
+          if (push) g.mark_active(q);
+        }
+        push_local<CTA>(g, sm, rc, nxt, nxt_n, push, sb + v, nb, ne, q);
+      }
+      for (unsigned lm = __ballot_sync(kFull, lng && sub == 0); lm; lm &= lm - 1) {
+        const int ld = __ffs(lm) - 1;
+        const uint32_t le = __shfl_sync(kFull, end, ld), lv = __shfl_sync(kFull, val, ld);
+        const uint32_t lq = __shfl_sync(kFull, q, ld);
+        const uint32_t lop = g.op(lq), lsb = g.sbase(lq);
+        for (uint32_t k0 = __shfl_sync(kFull, beg, ld); k0 < le; k0 += 32) {
+          const uint32_t k = k0 + lane;
+          bool push = false;
+          uint32_t v = 0, nb = 0, ne = 0;
+          if (k < le) {
+            v = ld_adj(g.colp(lq) + k);
+            const uint32_t nd = lv + ((OP == OP_BFSR) ? 1u : (needs_w<OP>(lop) ? static_cast<uint32_t>(ld_adj(g.wp(lq) + k)) : 0u));
+            const unsigned long long old = atomicMin(rc.ds + lsb + v, (static_cast<unsigned long long>(nd) << 32) | dsr);
+            nb = __ldg(g.rowp(lq) + v);
+            ne = __ldg(g.rowp(lq) + v + 1);
+            push = nd < static_cast<uint32_t>(old >> 32) && static_cast<uint32_t>(old) != dsr;
+            if constexpr (V::kBatched) {
+              if (push) g.mark_active(lq);
+            }
+          }
+          push_local<CTA>(g, sm, rc, nxt, nxt_n, push, lsb + v, nb, ne, lq);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // what the last sub-round discovered goes to the out-worklist
+  const uint32_t left = j > rc.local_rounds ? min(l_n[j % 3], C) : 0u;
+  if (left != 0) {
+    const uint32_t* const cur = (j & 1) ? half1 : half0;
+    if (tid == 0) {
+      sm.gbase = atomicAdd(rc.out.tail, left);
+      sm.round_pushes += left;
+    }
+    __syncthreads();
+    const uint32_t gb = sm.gbase;
+    for (uint32_t i = tid; i < left; i += CTA) {
+      if (gb + i < rc.out.cap) __stcg(rc.out.items + gb + i, cur[i]);
+      else set_err(rc.out.err, DERR_WL_OVERFLOW);
+      if (V::kBatched) g.mark(cur[3 * C + i], rc.ep);  // its query has out-worklist items left
+    }
+  }
+  if constexpr (V::kNear) {
+    if (g.lim != nullptr) flush_far<CTA>(g, sm, rc, 0u);
+  }
+  __syncthreads();
+}
+
 // ForAll over the in-worklist (Sec. 3.1): the first `chunk` tiles of CTA items
 // of each CTA are static (blockIdx-th span); the rest is grabbed dynamically
 // with one atomic per span, so small frontiers cost no contended atomic. A
 // frontier below one tile per CTA is spread over every CTA instead (below).
-template <uint32_t OP, int CTA, int RED, class V>
+template <uint32_t OP, int CTA, int RED, bool LOCAL, class V>
 __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t& edges,
                                            uint32_t& any_true, uint32_t& any_false) {
   const uint32_t span = CTA * rc.tn.chunk;
   const uint32_t static_end = gridDim.x * span;
   uint32_t gb = blockIdx.x * span;
+  if constexpr (LOCAL) {
+    if (rc.spread != 0 && rc.local_rounds != 0 && rc.in_n <= gridDim.x * CTA) {
+      local_round<OP, CTA>(g, sm, rc, edges);
+      return;
+    }
+  }
   if (rc.spread != 0 && rc.in_n <= gridDim.x * CTA) {
     // A frontier smaller than one tile per CTA is spread over the whole grid:
     // CTA b takes items b, b + grid, ..., dealt across its warps (slot s goes
@@ -1421,7 +1727,7 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
     // warp's chain of loads and atomics to one or two strips instead of
     // loading 128 items onto each of a few CTAs.
     const uint32_t slot = (threadIdx.x & 31u) * (CTA / 32) + (threadIdx.x >> 5);
-    if (blockIdx.x < rc.in_n) process_tile<OP, CTA, RED>(g, sm, rc, blockIdx.x + slot * gridDim.x, edges, any_true, any_false);
+    if (blockIdx.x < rc.in_n) process_tile<OP, CTA, RED, LOCAL>(g, sm, rc, blockIdx.x + slot * gridDim.x, edges, any_true, any_false);
     gb = rc.in_n;  // every item is taken
   }
   for (;;) {
@@ -1429,7 +1735,7 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
     for (uint32_t t = 0; t < rc.tn.chunk; ++t) {
       const uint32_t tb = gb + t * CTA;
       if (tb >= rc.in_n) break;
-      process_tile<OP, CTA, RED>(g, sm, rc, tb + threadIdx.x, edges, any_true, any_false);
+      process_tile<OP, CTA, RED, LOCAL>(g, sm, rc, tb + threadIdx.x, edges, any_true, any_false);
     }
     if (static_end >= rc.in_n) break;  // everything was covered by the static spans
     __syncthreads();
@@ -1437,7 +1743,7 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
     __syncthreads();
     gb = sm.grab_base;
   }
-  if constexpr (V::kBatched) {
+  if constexpr (V::kNear) {
     if (g.lim != nullptr && rc.far_in_n != 0) far_sweep<CTA>(g, sm, rc);
   }
   // CTA-local sub-rounds: expand the stage's newest items [lo, hi) here, with
@@ -1448,7 +1754,7 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
   // pushes the vertex again; the relaxation is label-correcting, so the fixed
   // point is the same. What is left unexpanded is flushed to the out-worklist.
   uint32_t lo = 0;
-  if (kPackedOp<OP> && rc.ds != nullptr && rc.local_rounds != 0) {
+  if (LOCAL && rc.local_rounds != 0) {
     RoundCtx lc = rc;
     for (uint32_t j = 1; j <= rc.local_rounds; ++j) {
       __syncthreads();
@@ -1458,12 +1764,15 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
       lc.in_n = hi - lo;
       lc.dsr = rc.dsr + j;
       for (uint32_t t = 0; t < hi - lo; t += CTA)
-        process_tile<OP, CTA, RED>(g, sm, lc, t + threadIdx.x, edges, any_true, any_false);
+        process_tile<OP, CTA, RED, LOCAL>(g, sm, lc, t + threadIdx.x, edges, any_true, any_false);
       lo = hi;
     }
   }
   __syncthreads();
   flush_stage<CTA>(sm, rc.out, lo);
+  if constexpr (V::kNear) {
+    if (g.lim != nullptr) flush_far<CTA>(g, sm, rc, 0u);
+  }
 }
 
 // ----------------------------------------------------------------------------- small-frontier round
@@ -1560,7 +1869,7 @@ __device__ __forceinline__ void broadcast_round(const SingleView<OP>& g, Smem<CT
       v[k] = 0;
       wt[k] = 0;
       sb[k] = 0;
-      op[k] = OP;
+      op[k] = base_op(OP);
       ov[k] = 0;
       if (e < hi) {
         // last list whose first edge is <= e (lists of degree 0 share offsets: the search skips them)
@@ -1573,7 +1882,7 @@ __device__ __forceinline__ void broadcast_round(const SingleView<OP>& g, Smem<CT
         const uint32_t edge = b_beg[a] + (e - b_off[a]);
         ov[k] = b_val[a];
         v[k] = ld_adj(g.col + edge);
-        if (needs_w<OP>(OP)) wt[k] = ld_adj(g.w + edge);
+        if (needs_w<OP>(base_op(OP))) wt[k] = ld_adj(g.w + edge);
         vmask |= 1u << k;
       }
     }
@@ -1818,7 +2127,7 @@ __device__ __forceinline__ void big_phase(const V& g, Smem<CTA>& sm, const Round
           if (rc.bdmin_next != nullptr) {
 #pragma unroll
             for (uint32_t k = 0; k < E; ++k)
-              note_pushes(rc.bdmin_next, g.slot(oqs[k]), (rr[k] == 1u && op[k] == OP_SSSP) ? ndv[k] : kInf);
+              if (rr[k] == 1u && op[k] == OP_SSSP) g.note(oqs[k], ndv[k]);
           }
         }
         push4<CTA>(sm, rc.out, f, sb[0] + v[0], sb[1] + v[1], sb[2] + v[2], sb[3] + v[3]);
@@ -2032,12 +2341,12 @@ __device__ __forceinline__ void split_far(const V& g, Smem<CTA>& sm, const Round
     uint32_t v = 0, d = kInf;
     if (i < far_n) {
       v = __ldcg(fin + i);
-      d = (OP == OP_SSSP && rc.ds != nullptr) ? static_cast<uint32_t>(__ldcg(rc.ds + v) >> 32) : __ldcg(g.state + v);
+      d = (base_op(OP) == OP_SSSP && rc.ds != nullptr) ? static_cast<uint32_t>(__ldcg(rc.ds + v) >> 32) : __ldcg(g.state + v);
     }
     // each vertex is on a phase's far list at most once and a split round
     // relaxes nothing, so with the packed words no round stamp is needed here
     const bool near = i < far_n && d >= lim_old && d < lim_new &&
-                      ((OP == OP_SSSP && rc.ds != nullptr) || atomicExch(g.stamp + v, rc.ep) != rc.ep);
+                      ((base_op(OP) == OP_SSSP && rc.ds != nullptr) || atomicExch(g.stamp + v, rc.ep) != rc.ep);
     const bool keep = i < far_n && d >= lim_new && atomicExch(rc.far_stamp + v, rc.phase) != rc.phase;
     push1<CTA>(sm, rc.out, near, v);
     push_far4<CTA>(sm, rc.far_out, keep ? 1u : 0u, v, 0u, 0u, 0u, d);
@@ -2058,7 +2367,7 @@ template <uint32_t OP>
 __device__ __forceinline__ void fill_state(uint32_t* state, uint32_t n, const uint32_t* srcs, uint32_t nsrc,
                                            uint32_t tid, uint32_t nthreads) {
   auto value = [&](uint32_t v) -> uint32_t {
-    if (OP == OP_CC) return v;
+    if (base_op(OP) == OP_CC) return v;
     uint32_t r = kInf;
 #pragma unroll
     for (uint32_t i = 0; i < 8; ++i) r = (i < nsrc && srcs[i] == v) ? 0u : r;
@@ -2195,7 +2504,8 @@ __device__ __forceinline__ void trace_end(unsigned long long* trace, uint32_t ca
 }
 
 // Iteration-outlined Iterate: every round in one cooperative launch.
-template <uint32_t OP, int CTA>
+// LOCAL: the launch has CTA-local sub-rounds (their code stays out of the other kernels).
+template <uint32_t OP, int CTA, bool LOCAL>
 __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& sm) {
   const unsigned long long t_start = p.trace ? globaltimer_ns() : 0ull;
   init_smem<CTA>(sm);
@@ -2222,11 +2532,11 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   if (p.init_state) {
     uint32_t srcs[8];
     uint32_t ns = 0;
-    const bool small = OP != OP_CC && p.init_items != nullptr && init_n <= 8;
+    const bool small = base_op(OP) != OP_CC && p.init_items != nullptr && init_n <= 8;
 #pragma unroll
     for (uint32_t i = 0; i < 8; ++i) srcs[i] = (small && i < init_n) ? __ldcg(p.init_items + i) : kInf;
     if (small) ns = init_n;
-    if ((OP == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) fill_packed(p.ds, p.n, srcs, ns, blockIdx.x * CTA + threadIdx.x, gridDim.x * CTA);
+    if ((base_op(OP) == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) fill_packed(p.ds, p.n, srcs, ns, blockIdx.x * CTA + threadIdx.x, gridDim.x * CTA);
     else fill_state<OP>(p.state, p.n, srcs, ns, blockIdx.x * CTA + threadIdx.x, gridDim.x * CTA);
     if constexpr (OP == OP_BFS) {
     // sources' out-degrees (every thread, the same few words): decide the fusion
@@ -2283,18 +2593,18 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
       if (threadIdx.x == 0) trace_phase_end(trace_phase(p.trace_ph, p.trace_cap, 0), 0);
     }
     }
-    if (OP != OP_CC && !small) {
+    if (base_op(OP) != OP_CC && !small) {
       ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
       if (ok) {
         for (uint32_t i = blockIdx.x * CTA + threadIdx.x; i < init_n; i += gridDim.x * CTA) {
           const uint32_t s = p.init_items ? __ldcg(p.init_items + i) : i;
           if (s >= p.n) continue;
-          if ((OP == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) __stcg(p.ds + s, 0ull);
+          if ((base_op(OP) == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) __stcg(p.ds + s, 0ull);
           else __stcg(p.state + s, 0u);
         }
       }
     }
-  } else if ((OP == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) {
+  } else if ((base_op(OP) == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) {
     // the caller's initial distances, round id 0
     for (uint32_t v = blockIdx.x * CTA + threadIdx.x; v < p.n; v += gridDim.x * CTA)
       __stcg(p.ds + v, static_cast<unsigned long long>(__ldcg(p.state + v)) << 32);
@@ -2354,10 +2664,10 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   }
   // small frontiers skip the big list (broadcast_round): BFS, SSSP and
   // min-label CC rounds (near-far included) without CTA-local sub-rounds
-  const bool bcast = p.bcast != 0 && (OP == OP_BFS || OP == OP_SSSP || OP == OP_CC) && p.local_rounds == 0;
+  const bool bcast = p.bcast != 0 && (OP == OP_BFS || base_op(OP) == OP_SSSP || base_op(OP) == OP_CC) && p.local_rounds == 0;
   // dense rounds: BFS, and SSSP on packed words, without near-far or sub-rounds
   const bool dense_ok = p.dense_div != 0 && !nf && p.local_rounds == 0 &&
-                        (OP == OP_BFS || (OP == OP_SSSP && p.ds != nullptr));
+                        (OP == OP_BFS || (base_op(OP) == OP_SSSP && p.ds != nullptr));
   // deferred expansion of long lists (SSSP on packed words, plain rounds)
   const bool defer = OP == OP_SSSP && p.defer_deg != 0 && p.ds != nullptr && !nf && p.local_rounds == 0 &&
                      p.dense_div == 0;
@@ -2383,9 +2693,9 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
     rc.mf = dopt ? &sm.mf_cta : nullptr;
     rc.row_ptr = p.row_ptr;
     rc.vis = OP == OP_BFS ? p.vis : nullptr;
-    rc.ds = (OP == OP_SSSP || OP == OP_BFSR) ? p.ds : nullptr;
+    rc.ds = (base_op(OP) == OP_SSSP || OP == OP_BFSR) ? p.ds : nullptr;
     rc.dsr = r * (p.local_rounds + 1u) + 1u;  // room for the sub-rounds' ids
-    rc.local_rounds = (OP == OP_SSSP || OP == OP_BFSR) ? p.local_rounds : 0u;
+    rc.local_rounds = LOCAL ? p.local_rounds : 0u;
     rc.local_items = nullptr;
     rc.spread = p.spread;
     if (defer && r > 0) {
@@ -2427,7 +2737,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
       // read at the start of the last round, before its barrier
       if (defer && blockIdx.x == 0) st->pmin[(r + 2) % 3] = 0;
     }
-    if (split) {
+    if (kNearFarOp<OP> && split) {
       split_far<OP, CTA>(g, sm, rc, fb ? p.far[1] : p.far[0], far_n, lim_old, limit);
     } else if (dopt && bottom_up) {
       // bottom-up round k reads the list round k - 1 left (count bu_n[(k - 1) % 3]) and
@@ -2444,7 +2754,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
     } else if (small_round) {
       broadcast_round<OP, CTA>(g, sm, rc, edges);
     } else {
-      round_body<OP, CTA, RED_NONE>(g, sm, rc, edges, dummy_t, dummy_f);
+      round_body<OP, CTA, RED_NONE, LOCAL>(g, sm, rc, edges, dummy_t, dummy_f);
     }
     if (dopt && threadIdx.x == 0 && sm.mf_cta) {
       atomicAdd(&st->mf[r % 3], sm.mf_cta);
@@ -2536,7 +2846,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
     }
     in_n = min(last_out, p.cap);
   }
-  if ((OP == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) {
+  if ((base_op(OP) == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) {
     // every round ended at a barrier that all CTAs passed: the words are final
     for (uint32_t v = blockIdx.x * CTA + threadIdx.x; v < p.n; v += gridDim.x * CTA)
       __stcg(p.state + v, static_cast<uint32_t>(__ldcg(p.ds + v) >> 32));
@@ -2812,7 +3122,7 @@ __device__ __forceinline__ void invoke_round(const KParams& p, const RoundArgs& 
   rc.local_rounds = 0;
   rc.local_items = nullptr;
   uint32_t edges = 0, any_true = 0, any_false = 0;
-  round_body<OP, CTA, RED>(g, sm, rc, edges, any_true, any_false);
+  round_body<OP, CTA, RED, false>(g, sm, rc, edges, any_true, any_false);
   const int t = __syncthreads_or(any_true != 0);
   const int f = __syncthreads_or(any_false != 0);
   const unsigned long long esum = cta_sum_u64<CTA>(sm, edges);
@@ -2841,8 +3151,8 @@ __device__ __forceinline__ void invoke_round(const KParams& p, const RoundArgs& 
 // the pending worklist left by the admission kernels (or by the previous
 // epoch); the launch stops when the worklist drains or after max_rounds
 // rounds (an epoch), leaving the pending items and their buffer in p.cont.
-template <int CTA>
-__device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA>& bs) {
+template <int CTA, bool NF, bool LOCAL>
+__device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA, NF>& bs) {
   Smem<CTA>& sm = bs.core;
   init_smem<CTA>(sm);
   const uint32_t nq = min(p.nq, static_cast<uint32_t>(kMaxBatchQueries));
@@ -2855,14 +3165,17 @@ __device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA>& 
   const uint32_t init_n = nq == 0 ? 0u : min(__ldcg(p.cont + 1), p.cap);
   // near-far (SSSP queries): limits in shared memory, advanced by delta after
   // every round in which the query pushed nothing to the out-worklist
-  const bool nf = p.delta != 0 && p.ds != nullptr;
+  const bool nf = NF && p.delta != 0 && p.ds != nullptr;
   // deferred expansion of long lists (SSSP queries, packed words, plain rounds)
   const bool bdefer = p.dmin != nullptr && p.defer_deg != 0 && p.ds != nullptr && !nf && p.local_rounds == 0;
   const uint32_t fcur0 = nf ? (__ldcg(p.cont + 2) & 1u) : 0u;
   uint32_t far_n = nf ? min(__ldcg(p.cont + 3), p.far_cap) : 0u;
   if (nf)
     for (uint32_t i = threadIdx.x; i < nq; i += CTA) bs.lim[i] = __ldcg(p.blim + __ldg(&p.desc[i].slot));
-  BatchView g{p.desc, bs.sbases, nq, p.state, p.stamp, bs.qbits, bs.qfar, nf ? bs.lim : nullptr, p.far_stamp};
+  BatchView<NF> g{p.desc, bs.sbases, nq, p.state, p.stamp, bs.qbits, bs.qfar, nf ? bs.lim : nullptr, p.far_stamp, bs.far_stage, &bs.far_n, bs.dmin};
+  if (threadIdx.x == 0) bs.far_n = 0;
+  if (!NF && bdefer)
+    for (uint32_t i = threadIdx.x; i < static_cast<uint32_t>(kMaxBatchQueries); i += CTA) bs.dmin[i] = kInf;
   if (threadIdx.x < kMaxBatchQueries / 32) {
     bs.qbits[threadIdx.x] = 0;
     bs.qfar[threadIdx.x] = 0;
@@ -2871,6 +3184,15 @@ __device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA>& 
   // fold this CTA's query bits into the round's global bitmaps (before a barrier)
   auto fold_marks = [&](uint32_t r) {
     __syncthreads();
+    if (!NF && bdefer && r >= 1) {
+      uint32_t* const next = p.dmin + ((r + 1u) % 3u) * kMaxBatchQueries;
+      for (uint32_t i = threadIdx.x; i < static_cast<uint32_t>(kMaxBatchQueries); i += CTA) {
+        const uint32_t d = bs.dmin[i];
+        if (d == kInf) continue;
+        atomicMax(next + i, ~d);  // stored complemented, so 0 means nothing pushed
+        bs.dmin[i] = kInf;
+      }
+    }
     for (uint32_t w = threadIdx.x; w < kMaxBatchQueries / 32; w += CTA) {
       const uint32_t bits = bs.qbits[w], fbits = bs.qfar[w];
       if (bits | fbits) {
@@ -2924,7 +3246,7 @@ __device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA>& 
     rc.vis = nullptr;
     rc.ds = p.ds;     // round ids are the global ones: admission writes id 0
     rc.dsr = rc.ep;
-    rc.local_rounds = p.ds != nullptr ? p.local_rounds : 0u;
+    rc.local_rounds = LOCAL && p.ds != nullptr ? p.local_rounds : 0u;
     rc.local_items = nullptr;
     rc.spread = p.spread;
     if (bdefer) {
@@ -2970,7 +3292,7 @@ __device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA>& 
       sm.round_pushes = 0;
       sm.big_appended = 0;
     }
-    round_body<OP_RUNTIME, CTA, RED_NONE>(g, sm, rc, edges, dummy_t, dummy_f);
+    round_body<OP_RUNTIME, CTA, RED_NONE, LOCAL>(g, sm, rc, edges, dummy_t, dummy_f);
     fold_marks(r);
     ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns, p.big.cap != 0);
     if (!ok) break;

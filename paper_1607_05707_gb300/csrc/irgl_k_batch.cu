@@ -4,10 +4,11 @@
 
 namespace irgl {
 
-template <int CTA>
+// NF: near-far may be on; LOCAL: CTA-local sub-rounds (with or without near-far).
+template <int CTA, bool NF, bool LOCAL>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_batch_iterate(BParams p) {
-  __shared__ BatchSmem<CTA> bs;
-  iterate_batch<CTA>(p, bs);
+  __shared__ BatchSmem<CTA, NF> bs;
+  iterate_batch<CTA, NF, LOCAL>(p, bs);
 }
 
 __global__ void __launch_bounds__(256) k_batch_fill(AdmitParams a) { admit_fill(a); }
@@ -36,7 +37,9 @@ cudaError_t launch_b(uint32_t grid, const BParams& p, cudaStream_t s) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA>, p);
+  if (p.local_rounds != 0) return cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, true, true>, p);
+  return p.delta != 0 ? cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, true, false>, p)
+                      : cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, false, false>, p);
 }
 
 }  // namespace
@@ -51,14 +54,19 @@ cudaError_t launch_batch_iterate(uint32_t cta, uint32_t grid, const BParams& p, 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t occupancy_batch(uint32_t cta, int* nb) {
+template <bool NF, bool LOCAL>
+cudaError_t occ_b(uint32_t cta, int* nb) {
   switch (cta) {
-    case 128: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<128>, 128, 0);
-    case 256: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<256>, 256, 0);
-    case 512: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<512>, 512, 0);
-    case 1024: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<1024>, 1024, 0);
+    case 128: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<128, NF, LOCAL>, 128, 0);
+    case 256: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<256, NF, LOCAL>, 256, 0);
+    case 512: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<512, NF, LOCAL>, 512, 0);
+    case 1024: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_batch_iterate<1024, NF, LOCAL>, 1024, 0);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t occupancy_batch(uint32_t cta, bool near_far, bool local, int* nb) {
+  return local ? occ_b<true, true>(cta, nb) : near_far ? occ_b<true, false>(cta, nb) : occ_b<false, false>(cta, nb);
 }
 
 cudaError_t launch_extract_values(const unsigned long long* ds, uint32_t* out, uint64_t n, uint32_t grid,

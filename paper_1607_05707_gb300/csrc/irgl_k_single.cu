@@ -5,10 +5,10 @@
 
 namespace irgl {
 
-template <uint32_t OP, int CTA>
+template <uint32_t OP, int CTA, bool LOCAL>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_iterate(KParams p) {
   __shared__ Smem<CTA> sm;
-  iterate_persistent<OP, CTA>(p, sm);
+  iterate_persistent<OP, CTA, LOCAL>(p, sm);
 }
 
 // Pointer-jumping CC: one CTA per SM, its vertex block in dynamic shared memory.
@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(kUfCta, 1) k_cc_jump(KParams p) {
 
 namespace {
 
-template <uint32_t OP, int CTA>
+template <uint32_t OP, int CTA, bool LOCAL>
 cudaError_t launch_one(uint32_t grid, const KParams& p, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -32,16 +32,16 @@ cudaError_t launch_one(uint32_t grid, const KParams& p, cudaStream_t s) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_iterate<OP, CTA>, p);
+  return cudaLaunchKernelEx(&cfg, k_iterate<OP, CTA, LOCAL>, p);
 }
 
-template <uint32_t OP>
+template <uint32_t OP, bool LOCAL = false>
 cudaError_t launch_op(uint32_t cta, uint32_t grid, const KParams& p, cudaStream_t s) {
   switch (cta) {
-    case 128: return launch_one<OP, 128>(grid, p, s);
-    case 256: return launch_one<OP, 256>(grid, p, s);
-    case 512: return launch_one<OP, 512>(grid, p, s);
-    case 1024: return launch_one<OP, 1024>(grid, p, s);
+    case 128: return launch_one<OP, 128, LOCAL>(grid, p, s);
+    case 256: return launch_one<OP, 256, LOCAL>(grid, p, s);
+    case 512: return launch_one<OP, 512, LOCAL>(grid, p, s);
+    case 1024: return launch_one<OP, 1024, LOCAL>(grid, p, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -98,13 +98,13 @@ cudaError_t occ_prefer_l1(K kern, int cta, int* nb) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, kern, cta, 0);
 }
 
-template <uint32_t OP>
+template <uint32_t OP, bool LOCAL = false>
 cudaError_t occ_op(uint32_t cta, int* nb) {
   switch (cta) {
-    case 128: return occ_prefer_l1(k_iterate<OP, 128>, 128, nb);
-    case 256: return occ_prefer_l1(k_iterate<OP, 256>, 256, nb);
-    case 512: return occ_prefer_l1(k_iterate<OP, 512>, 512, nb);
-    case 1024: return occ_prefer_l1(k_iterate<OP, 1024>, 1024, nb);
+    case 128: return occ_prefer_l1(k_iterate<OP, 128, LOCAL>, 128, nb);
+    case 256: return occ_prefer_l1(k_iterate<OP, 256, LOCAL>, 256, nb);
+    case 512: return occ_prefer_l1(k_iterate<OP, 512, LOCAL>, 512, nb);
+    case 1024: return occ_prefer_l1(k_iterate<OP, 1024, LOCAL>, 1024, nb);
   }
   return cudaErrorInvalidValue;
 }
@@ -117,7 +117,10 @@ cudaError_t launch_iterate(uint32_t op, uint32_t cta, uint32_t grid, const KPara
     case OP_SSSP: return launch_op<OP_SSSP>(cta, grid, p, s);
     case OP_CC: return launch_op<OP_CC>(cta, grid, p, s);
     case OP_CCJ: return launch_cc_jump(cta, grid, p, s);
-    case OP_BFSR: return launch_op<OP_BFSR>(cta, grid, p, s);
+    case OP_BFSR: return launch_op<OP_BFSR, true>(cta, grid, p, s);
+    case OP_SSSPL: return launch_op<OP_SSSP, true>(cta, grid, p, s);
+    case OP_SSSPF: return launch_op<OP_SSSPF>(cta, grid, p, s);
+    case OP_CCF: return launch_op<OP_CCF>(cta, grid, p, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -128,7 +131,10 @@ cudaError_t occupancy_iterate(uint32_t op, uint32_t cta, int* nb) {
     case OP_SSSP: return occ_op<OP_SSSP>(cta, nb);
     case OP_CC: return occ_op<OP_CC>(cta, nb);
     case OP_CCJ: return occ_cc_jump(nb);
-    case OP_BFSR: return occ_op<OP_BFSR>(cta, nb);
+    case OP_BFSR: return occ_op<OP_BFSR, true>(cta, nb);
+    case OP_SSSPL: return occ_op<OP_SSSP, true>(cta, nb);
+    case OP_SSSPF: return occ_op<OP_SSSPF>(cta, nb);
+    case OP_CCF: return occ_op<OP_CCF>(cta, nb);
   }
   return cudaErrorInvalidValue;
 }

@@ -25,7 +25,8 @@ cudaError_t launch_wl_append(uint32_t* items, uint32_t* tail, uint32_t cap, cons
 
 // Batched multi-query Iterate (cooperative) and query admission.
 cudaError_t launch_batch_iterate(uint32_t cta, uint32_t grid, const BParams& p, cudaStream_t s);
-cudaError_t occupancy_batch(uint32_t cta, int* blocks_per_sm);
+// near_far, local: the launch has a delta, CTA-local sub-rounds
+cudaError_t occupancy_batch(uint32_t cta, bool near_far, bool local, int* blocks_per_sm);
 cudaError_t launch_admit(const AdmitParams& a, uint32_t grid, cudaStream_t s);
 // out[i] = value half of the packed arena word ds[i], i < n.
 cudaError_t launch_extract_values(const unsigned long long* ds, uint32_t* out, uint64_t n, uint32_t grid,

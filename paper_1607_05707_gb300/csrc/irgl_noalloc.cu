@@ -49,7 +49,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocS
 
 __global__ void __launch_bounds__(kNoAllocCta, MinBlocks<kNoAllocCta>::value) k_bfs_noalloc(KParams p) {
   __shared__ Smem<kNoAllocCta> sm;
-  iterate_persistent<OP_BFS, kNoAllocCta>(p, sm);
+  iterate_persistent<OP_BFS, kNoAllocCta, false>(p, sm);
 }
 
 struct DeviceSetup {

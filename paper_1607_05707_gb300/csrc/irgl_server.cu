@@ -860,7 +860,7 @@ irgl_status irgl_server_create(irgl_ctx* ctx, const irgl_server_config* cfg, irg
   if (e == cudaSuccess) e = cudaMemsetAsync(s->qlast, 0, sizeof(uint32_t) * S, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   int nb = 0;
-  if (e == cudaSuccess) e = occupancy_batch(t.cta_size, &nb);
+  if (e == cudaSuccess) e = occupancy_batch(t.cta_size, s->blim != nullptr, s->sub_rounds != 0, &nb);
   if (e != cudaSuccess || nb <= 0) {
     server_free(s);
     delete s;
