@@ -1061,8 +1061,10 @@ __device__ __forceinline__ bool group_edges(const V& g, Smem<CTA>& sm, const Rou
     }
     any |= (fn | ff) != 0;
     if (GROUP == CTA) {
-      // the predicate is taken at the barrier, when every warp's pushes are in
-      if (__syncthreads_or(sm.stage_n >= static_cast<uint32_t>(Smem<CTA>::kStage / 2))) flush_stage<CTA>(sm, rc.out);
+      // the predicate is taken at the barrier, when every warp's pushes are in; a
+      // sub-round reads its items from the stage, and no flush may move them under it
+      if (__syncthreads_or(rc.local_items == nullptr && sm.stage_n >= static_cast<uint32_t>(Smem<CTA>::kStage / 2)))
+        flush_stage<CTA>(sm, rc.out);
     }
   }
   scalar(b + rank, end);
