@@ -96,7 +96,9 @@ typedef struct {
                              value (distance, label) >= the current limit wait on a far list until
                              the rounds below the limit drain; 0 = plain rounds (every improvement
                              is pushed). CC with delta = 1 floods the smallest label first, so
-                             each vertex mostly takes its final label once. Batches and servers:
+                             each vertex mostly takes its final label once. SSSP on a graph of short
+                             lists (m <= 6 n, none at the degree thresholds) takes CTA-local sub-rounds
+                             in its sparse rounds by itself (up to 16 worklist entries per vertex). Batches and servers:
                              per-query near-far for their SSSP queries (below) */
   uint32_t defer_deg;     /* persistent SSSP with plain rounds (delta = 0, no sub-rounds): a popped
                              vertex with at least defer_deg out-edges whose distance is above the

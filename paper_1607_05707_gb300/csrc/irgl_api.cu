@@ -817,11 +817,20 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   const bool packed = (k == IRGL_SSSP || (k == IRGL_BFS && use_local)) && mode == IRGL_PERSISTENT &&
                       !(t.flags & IRGL_TUNE_NO_PACKED);
   const bool far = (k == IRGL_SSSP || k == IRGL_CC) && mode == IRGL_PERSISTENT && t.delta != 0;
+  // Near-far SSSP on a graph of short lists takes sub-rounds in its sparse rounds by
+  // itself: a frontier of a mesh or road network (m / n of 2 to 5) advances a hop per
+  // round; one of a power-law graph reaches everything in a few dozen rounds and only
+  // rescans (R-MAT of 2^18 vertices, 4 edges each: 298 us plain, 383 with sub-rounds), so
+  // a long list, known here or met on the device, turns them off. Fewer of them on
+  // larger graphs, whose worklists (n entries per sub-round id) would pass 0.5 GB each.
+  const bool short_lists = g->m <= 6ull * g->n && (g->max_deg == 0xFFFFFFFFu || g->max_deg < std::min(t.warp_thresh, t.cta_thresh));
+  const uint32_t near_rounds = !(far && packed && k == IRGL_SSSP && short_lists) ? 0u
+                               : g->n <= (1u << 23) ? 15u : g->n <= (1u << 25) ? 3u : 0u;
   // a vertex can be pushed once per sub-round: worklists of n * (sub-rounds + 1)
-  s = ensure_workspace(ctx, g->n, k != IRGL_BFS, far, vis, packed, use_local ? sub_rounds + 1u : 1u);
+  s = ensure_workspace(ctx, g->n, k != IRGL_BFS, far, vis, packed, (use_local ? sub_rounds : near_rounds) + 1u);
   if (s != IRGL_OK) return s;
   const uint32_t op = use_local ? (k == IRGL_BFS ? OP_BFSR : OP_SSSPL)
-                      : far ? (k == IRGL_SSSP ? OP_SSSPF : OP_CCF) : op_of(k);
+                      : far ? (k == IRGL_SSSP ? (near_rounds ? OP_SSSPFL : OP_SSSPF) : OP_CCF) : op_of(k);
   if (k == IRGL_CC_JUMP) t.cta_size = kUfCta;  // its vertex blocks fill an SM's shared memory: one CTA each
   if (k == IRGL_CC_JUMP && mode != IRGL_PERSISTENT)
     return fail(IRGL_ERR_UNSUPPORTED, "pointer-jumping CC runs only as a persistent Iterate");
@@ -853,12 +862,12 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
     p.bu_list[0] = ctx->ws_bu[0];
     p.bu_list[1] = ctx->ws_bu[1];
   }
-  if (use_local) {
-    p.local_rounds = sub_rounds;
+  if (use_local || near_rounds) {
+    p.local_rounds = use_local ? sub_rounds : near_rounds;
     p.diropt = 0;
     // round r stamps with ids r * (sub-rounds + 1) + 1 .. (r + 1) * (sub-rounds + 1):
     // stop before they would wrap to 0, the "on no worklist" stamp
-    p.max_rounds = std::min(p.max_rounds, 0xFFFFFFFFu / (sub_rounds + 1u) - 1u);
+    p.max_rounds = std::min(p.max_rounds, 0xFFFFFFFFu / (p.local_rounds + 1u) - 1u);
   }
   irgl_stats local;
   std::memset(&local, 0, sizeof(local));

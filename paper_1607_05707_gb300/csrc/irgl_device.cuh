@@ -38,14 +38,14 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // since a vertex can be reached there before its level is final.
 // OP_SSSPF, OP_CCF: SSSP and min-label CC with the near-far schedule, kernels of
 // their own: its lists and limits kept in registers beside the plain rounds' code
-// made the plain SSSP kernel spill (112 bytes of spill loads, 20 without). OP_SSSPL: launch table entry of the
-// SSSP kernel with CTA-local sub-rounds (LOCAL below).
+// made the plain SSSP kernel spill (112 bytes of spill loads, 20 without). OP_SSSPL, OP_SSSPFL: launch table entries of the
+// SSSP and near-far SSSP kernels with CTA-local sub-rounds (LOCAL below).
 enum : uint32_t { OP_BFS = 0, OP_SSSP = 1, OP_CC = 2, OP_RUNTIME = 3, OP_CCJ = 4, OP_BFSR = 5, OP_SSSPL = 6, OP_SSSPF = 7,
-                  OP_CCF = 8 };
+                  OP_CCF = 8, OP_SSSPFL = 9 };
 
 // The operator an id stands for.
 __host__ __device__ constexpr uint32_t base_op(uint32_t op) {
-  return op == OP_SSSPF || op == OP_SSSPL ? static_cast<uint32_t>(OP_SSSP) : op == OP_CCF ? static_cast<uint32_t>(OP_CC) : op;
+  return op == OP_SSSPF || op == OP_SSSPL || op == OP_SSSPFL ? static_cast<uint32_t>(OP_SSSP) : op == OP_CCF ? static_cast<uint32_t>(OP_CC) : op;
 }
 
 // Operators whose values are scheduled near-far (smallest first): SSSP distances
@@ -1516,6 +1516,16 @@ __device__ __forceinline__ void push_local(const V& g, Smem<CTA>& sm, const Roun
   }
 }
 
+// Near-far SSSP (one query): its rounds take the sub-rounds by themselves, up to
+// kNearLocal items per CTA. Improvements at or above the limit are staged for the far
+// list in kLocalFar words (one atomic per CTA and round instead of one per pushing
+// warp, whose answer the next sub-round would wait for). A CTA whose entries have
+// grown past kNearGrow + twice what it started with leaves the rest to the grid: on a
+// mesh a frontier grows by a few vertices per hop, on a power-law graph by orders.
+// 1021 x 1031 mesh, delta 1024, a source near a corner: 1883 rounds of 7.7 us and 16.4 ms
+// before, 4.6 ms now; 300 x 310: 4.6 and 1.15 ms; R-MAT of 2^18 vertices unchanged.
+constexpr uint32_t kNearLocal = 64, kNearGrow = 64, kLocalFar = 512;
+
 template <uint32_t OP, int CTA, class V>
 __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t& edges) {
   constexpr uint32_t C = LocalBuf<CTA, V>::kCap;
@@ -1526,6 +1536,9 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
   uint32_t* const half1 = sm.stage + LocalBuf<CTA, V>::kFields * C;
   const uint32_t m = rc.in_n > blockIdx.x ? (rc.in_n - blockIdx.x - 1u) / gridDim.x + 1u : 0u;  // <= CTA
   if (tid < 3) l_n[tid] = tid == 0 ? m : 0u;
+  __shared__ uint32_t s_far[kNearFarOp<OP> ? kLocalFar : 1u];
+  __shared__ uint32_t s_far_n;
+  if (kNearFarOp<OP> && tid == 0) s_far_n = 0;
   __syncthreads();
   if (tid < m) {
     const uint32_t idx = blockIdx.x + tid * gridDim.x;
@@ -1579,6 +1592,21 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
   }
   __syncthreads();
   const uint32_t split = min(rc.tn.warp_thresh, rc.tn.cta_thresh);  // as a frontier below one tile per CTA splits
+  // near-far: v's distance fell to nd, at or above the limit (at most once per phase)
+  auto push_far_local = [&](bool far, uint32_t v, uint32_t nd) {
+    const bool want = far && atomicExch(rc.far_stamp + v, rc.phase) != rc.phase;
+    const unsigned fm = __ballot_sync(kFull, want);
+    if (fm == 0) return;
+    const int ld = __ffs(fm) - 1;
+    const uint32_t cnt = __popc(fm);
+    uint32_t base = 0;
+    if (lane == static_cast<uint32_t>(ld)) base = atomicAdd(&s_far_n, cnt);
+    base = __shfl_sync(kFull, base, ld);
+    const uint32_t pos = base + __popc(fm & lanemask_lt());
+    if (want) atomicMin(&sm.far_min_cta, nd);
+    if (want && pos < kLocalFar) s_far[kNearFarOp<OP> ? pos : 0u] = v;
+    if (base + cnt > kLocalFar) push_far4<CTA>(sm, rc.far_out, want && pos >= kLocalFar ? 1u : 0u, v, 0u, 0u, 0u, nd);
+  };
   uint32_t j = 0;
   for (; j <= rc.local_rounds; ++j) {
     const uint32_t n = min(l_n[j % 3], C);
@@ -1644,7 +1672,9 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
         uint32_t nb = 0, ne = 0;
         const uint32_t nd = val + add, v = c;
         if (mine) {
-          old = atomicMin(rc.ds + sb + v, (static_cast<unsigned long long>(nd) << 32) | dsr);
+          // a far improvement stamps 0: the vertex is on no out-worklist (see decide_n)
+          old = atomicMin(rc.ds + sb + v, (static_cast<unsigned long long>(nd) << 32) |
+                                              (kNearFarOp<OP> && nd >= rc.limit ? 0u : dsr));
           nb = __ldg(rowp + v);
           ne = __ldg(rowp + v + 1);
         }
@@ -1652,11 +1682,13 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
           c = __ldg(col + k + 4u);
           if (nw) add = static_cast<uint32_t>(__ldg(w + k + 4u));
         }
-        const bool push = mine && nd < static_cast<uint32_t>(old >> 32) && static_cast<uint32_t>(old) != dsr;
+        const bool better = mine && nd < static_cast<uint32_t>(old >> 32);
+        const bool push = better && !(kNearFarOp<OP> && nd >= rc.limit) && static_cast<uint32_t>(old) != dsr;
         if constexpr (V::kBatched) {
           if (push) g.mark_active(q);
         }
         push_local<CTA>(g, sm, rc, nxt, nxt_n, push, sb + v, nb, ne, q);
+        if constexpr (kNearFarOp<OP>) push_far_local(better && nd >= rc.limit, v, nd);
       }
       for (unsigned lm = __ballot_sync(kFull, lng && sub == 0); lm; lm &= lm - 1) {
         const int ld = __ffs(lm) - 1;
@@ -1665,27 +1697,37 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
         const uint32_t lop = g.op(lq), lsb = g.sbase(lq);
         for (uint32_t k0 = __shfl_sync(kFull, beg, ld); k0 < le; k0 += 32) {
           const uint32_t k = k0 + lane;
-          bool push = false;
-          uint32_t v = 0, nb = 0, ne = 0;
+          bool push = false, far = false;
+          uint32_t v = 0, nb = 0, ne = 0, nd = 0;
           if (k < le) {
             v = ld_adj(g.colp(lq) + k);
-            const uint32_t nd = lv + ((OP == OP_BFSR) ? 1u : (needs_w<OP>(lop) ? static_cast<uint32_t>(ld_adj(g.wp(lq) + k)) : 0u));
-            const unsigned long long old = atomicMin(rc.ds + lsb + v, (static_cast<unsigned long long>(nd) << 32) | dsr);
+            nd = lv + ((OP == OP_BFSR) ? 1u : (needs_w<OP>(lop) ? static_cast<uint32_t>(ld_adj(g.wp(lq) + k)) : 0u));
+            const bool above = kNearFarOp<OP> && nd >= rc.limit;
+            const unsigned long long old =
+                atomicMin(rc.ds + lsb + v, (static_cast<unsigned long long>(nd) << 32) | (above ? 0u : dsr));
             nb = __ldg(g.rowp(lq) + v);
             ne = __ldg(g.rowp(lq) + v + 1);
-            push = nd < static_cast<uint32_t>(old >> 32) && static_cast<uint32_t>(old) != dsr;
+            const bool better = nd < static_cast<uint32_t>(old >> 32);
+            far = better && above;
+            push = better && !above && static_cast<uint32_t>(old) != dsr;
             if constexpr (V::kBatched) {
               if (push) g.mark_active(lq);
             }
           }
           push_local<CTA>(g, sm, rc, nxt, nxt_n, push, lsb + v, nb, ne, lq);
+          if constexpr (kNearFarOp<OP>) push_far_local(far, v, nd);
         }
       }
     }
     __syncthreads();
+    if (kNearFarOp<OP> && l_n[(j + 1) % 3] > kNearGrow + 2u * m) {  // CTA-uniform: read after the barrier
+      ++j;
+      break;
+    }
   }
   // what the last sub-round discovered goes to the out-worklist
-  const uint32_t left = j > rc.local_rounds ? min(l_n[j % 3], C) : 0u;
+  // (or, near-far, of the sub-round that grew too far; 0 when the loop ran dry)
+  const uint32_t left = min(l_n[j % 3], C);
   if (left != 0) {
     const uint32_t* const cur = (j & 1) ? half1 : half0;
     if (tid == 0) {
@@ -1703,6 +1745,18 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
   if constexpr (V::kNear) {
     if (g.lim != nullptr) flush_far<CTA>(g, sm, rc, 0u);
   }
+  if constexpr (kNearFarOp<OP>) {
+    __syncthreads();
+    const uint32_t n = min(s_far_n, kLocalFar);
+    if (n != 0) {
+      if (tid == 0) sm.gbase = atomicAdd(rc.far_out.tail, n);
+      __syncthreads();
+      for (uint32_t i = tid; i < n; i += CTA) {
+        if (sm.gbase + i < rc.far_out.cap) __stcg(rc.far_out.items + sm.gbase + i, s_far[i]);
+        else set_err(rc.far_out.err, DERR_WL_OVERFLOW);
+      }
+    }
+  }
   __syncthreads();
 }
 
@@ -1717,7 +1771,7 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
   const uint32_t static_end = gridDim.x * span;
   uint32_t gb = blockIdx.x * span;
   if constexpr (LOCAL) {
-    if (rc.spread != 0 && rc.local_rounds != 0 && rc.in_n <= gridDim.x * CTA) {
+    if (rc.spread != 0 && rc.local_rounds != 0 && rc.in_n <= gridDim.x * (kNearFarOp<OP> ? kNearLocal : CTA)) {
       local_round<OP, CTA>(g, sm, rc, edges);
       return;
     }
@@ -1756,7 +1810,7 @@ __device__ __forceinline__ void round_body(const V& g, Smem<CTA>& sm, const Roun
   // pushes the vertex again; the relaxation is label-correcting, so the fixed
   // point is the same. What is left unexpanded is flushed to the out-worklist.
   uint32_t lo = 0;
-  if (LOCAL && rc.local_rounds != 0) {
+  if (LOCAL && !kNearFarOp<OP> && rc.local_rounds != 0) {
     RoundCtx lc = rc;
     for (uint32_t j = 1; j <= rc.local_rounds; ++j) {
       __syncthreads();
@@ -2666,7 +2720,11 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   }
   // small frontiers skip the big list (broadcast_round): BFS, SSSP and
   // min-label CC rounds (near-far included) without CTA-local sub-rounds
-  const bool bcast = p.bcast != 0 && (OP == OP_BFS || base_op(OP) == OP_SSSP || base_op(OP) == OP_CC) && p.local_rounds == 0;
+  // near-far sub-rounds end for good with the first list long enough for the big list:
+  // a graph that has those is not the mesh they are for (borrowed graphs' degrees are
+  // not known to the host)
+  bool near_local = LOCAL && kNearFarOp<OP>;
+  const bool bcast_ok = p.bcast != 0 && (OP == OP_BFS || base_op(OP) == OP_SSSP || base_op(OP) == OP_CC);
   // dense rounds: BFS, and SSSP on packed words, without near-far or sub-rounds
   const bool dense_ok = p.dense_div != 0 && !nf && p.local_rounds == 0 &&
                         (OP == OP_BFS || (base_op(OP) == OP_SSSP && p.ds != nullptr));
@@ -2697,9 +2755,10 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
     rc.vis = OP == OP_BFS ? p.vis : nullptr;
     rc.ds = (base_op(OP) == OP_SSSP || OP == OP_BFSR) ? p.ds : nullptr;
     rc.dsr = r * (p.local_rounds + 1u) + 1u;  // room for the sub-rounds' ids
-    rc.local_rounds = LOCAL ? p.local_rounds : 0u;
+    rc.local_rounds = LOCAL && (!kNearFarOp<OP> || near_local) ? p.local_rounds : 0u;
     rc.local_items = nullptr;
     rc.spread = p.spread;
+    const bool bcast = bcast_ok && rc.local_rounds == 0;
     if (defer && r > 0) {
       // the smallest distance pushed for this round (complete at the last barrier)
       const uint32_t pm = __ldcg(&st->pmin[r % 3]);
@@ -2779,6 +2838,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
       ph[3] = (sm.pub_flags & kRelBigFlag) ? sm.pub_big : 0ull;
     }
     if (sm.pub_flags & kRelBigFlag) {
+      near_local = false;
       big_phase<OP, CTA>(g, sm, rc, sm.pub_big);
       if (nf && threadIdx.x == 0 && sm.far_min_cta != kInf) atomicMax(&st->far_min[ftarget], ~sm.far_min_cta);
       if (dopt && threadIdx.x == 0 && sm.mf_cta) {

@@ -120,6 +120,7 @@ cudaError_t launch_iterate(uint32_t op, uint32_t cta, uint32_t grid, const KPara
     case OP_BFSR: return launch_op<OP_BFSR, true>(cta, grid, p, s);
     case OP_SSSPL: return launch_op<OP_SSSP, true>(cta, grid, p, s);
     case OP_SSSPF: return launch_op<OP_SSSPF>(cta, grid, p, s);
+    case OP_SSSPFL: return launch_op<OP_SSSPF, true>(cta, grid, p, s);
     case OP_CCF: return launch_op<OP_CCF>(cta, grid, p, s);
   }
   return cudaErrorInvalidValue;
@@ -134,6 +135,7 @@ cudaError_t occupancy_iterate(uint32_t op, uint32_t cta, int* nb) {
     case OP_BFSR: return occ_op<OP_BFSR, true>(cta, nb);
     case OP_SSSPL: return occ_op<OP_SSSP, true>(cta, nb);
     case OP_SSSPF: return occ_op<OP_SSSPF>(cta, nb);
+    case OP_SSSPFL: return occ_op<OP_SSSPF, true>(cta, nb);
     case OP_CCF: return occ_op<OP_CCF>(cta, nb);
   }
   return cudaErrorInvalidValue;
