@@ -350,6 +350,8 @@ __device__ __forceinline__ uint4 ld_adj4(const uint4* p) { return __ldg(p); }
 __device__ __forceinline__ int4 ld_adj4(const int4* p) { return __ldg(p); }
 #endif
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" : : "l"(p)); }
+
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
   const uint32_t lane = threadIdx.x & 31;
 #pragma unroll
@@ -1634,6 +1636,7 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
       const uint32_t* const rowp = g.rowp(q);
       const uint32_t sb = g.sbase(q);
       const bool nw = valid && needs_w<OP>(op);
+      const uint32_t nv = g.nverts(q);
       uint32_t c = beg + sub < end ? __ldg(col + beg + sub) : 0u;
       uint32_t add = (OP == OP_BFSR) ? 1u : (nw && beg + sub < end ? static_cast<uint32_t>(__ldg(w + beg + sub)) : 0u);
       // the value the out-edges start from (a batched BFS item: the level they assign)
@@ -1686,6 +1689,14 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
         const bool push = better && !(kNearFarOp<OP> && nd >= rc.limit) && static_cast<uint32_t>(old) != dsr;
         if constexpr (V::kBatched) {
           if (push) g.mark_active(q);
+        }
+        if (push) {
+          // what the next sub-rounds read if ids have locality: v's columns, and the words
+          // a line further on either side (4096^2 mesh BFS 12.25 -> 11.5 ms, columns alone
+          // 11.77, words alone 11.90)
+          if (nb < ne) prefetch_l2(col + nb);
+          if (v >= 16u) prefetch_l2(rc.ds + sb + v - 16u);
+          if (v + 16u < nv) prefetch_l2(rc.ds + sb + v + 16u);
         }
         push_local<CTA>(g, sm, rc, nxt, nxt_n, push, sb + v, nb, ne, q);
         if constexpr (kNearFarOp<OP>) push_far_local(better && nd >= rc.limit, v, nd);
