@@ -126,6 +126,29 @@ irgl_status read_status(irgl_ctx* ctx, DevStatus* out) {
   return IRGL_OK;
 }
 
+// Wait for the launch that was given ctx->rec. Its record in place: the pinned mirror
+// gets the outcome without a copy. Otherwise (an error, a launch that ended early, an
+// epoch about to wrap) the status block is read, and the edge counter cleared behind it.
+irgl_status wait_launch(irgl_ctx* ctx) {
+  const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "launch");
+  const volatile HostRec* r = ctx->rec;
+  if (r->seq == ctx->rec_seq && r->err == DERR_NONE && r->epoch <= 0xF0000000u) {
+    DevStatus& h = *ctx->st_host;
+    h.err = DERR_NONE;
+    h.rounds = r->rounds;
+    h.last_out = r->last_out;
+    h.epoch = r->epoch;
+    h.edges = r->edges;
+    return IRGL_OK;
+  }
+  const unsigned long long taken = r->seq == ctx->rec_seq ? r->edges : 0ull;
+  const irgl_status s = read_status(ctx, nullptr);
+  ctx->st_host->edges += taken;  // what the kernel took out of the counter for its record
+  if (s == IRGL_OK) cudaMemsetAsync(&ctx->st->edges, 0, sizeof(unsigned long long), ctx->stream);
+  return s;
+}
+
 void reset_status(irgl_ctx* ctx) {
   // Clear counters and errors. Stamps may hold any epoch used so far, so they
   // are cleared too and the epoch restarts at 1.
@@ -349,7 +372,12 @@ irgl_status irgl_ctx_create(int device, void* cuda_stream, irgl_ctx** out) {
   e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (e == cudaSuccess) e = cudaMalloc(&ctx->st, sizeof(DevStatus));
-  if (e == cudaSuccess) e = cudaMallocHost(&ctx->st_host, sizeof(DevStatus));
+  // pinned: the status mirror and, a line further, the launch record
+  if (e == cudaSuccess) e = cudaMallocHost(&ctx->st_host, sizeof(DevStatus) + sizeof(HostRec));
+  if (e == cudaSuccess) {
+    ctx->rec = reinterpret_cast<HostRec*>(ctx->st_host + 1);
+    std::memset(ctx->rec, 0, sizeof(HostRec));
+  }
   if (e != cudaSuccess) {
     irgl_ctx_destroy(ctx);
     return cuda_fail(e, "context setup");
@@ -799,7 +827,7 @@ irgl_status irgl_invoke(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workli
 
 irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_worklist* initial, uint32_t* state_dev,
                          irgl_mode mode, const irgl_tuning* tin, uint32_t max_rounds, irgl_stats* stats,
-                         bool sync) {
+                         bool sync, bool record) {
   if (!ctx || !g || !state_dev) return fail(IRGL_ERR_INVALID_ARG, "NULL argument");
   if (mode != IRGL_PER_LAUNCH && mode != IRGL_PERSISTENT) return fail(IRGL_ERR_INVALID_ARG, "unknown mode");
   irgl_status s = check_kernel_graph(k, g);
@@ -839,6 +867,14 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   p.init_count = initial ? initial->tail : nullptr;
   p.init_cap = initial ? initial->cap : 0;
   p.max_rounds = max_rounds ? max_rounds : 0xFFFFFFFFu;
+  if (!initial && ctx->isrc_n) {
+    p.isrc_n = ctx->isrc_n;
+    std::memcpy(p.isrc, ctx->isrc, sizeof(p.isrc));
+  }
+  if (mode == IRGL_PERSISTENT && (sync || record)) {
+    p.rec = ctx->rec;
+    p.rec_seq = ++ctx->rec_seq;
+  }
   if (vis) p.vis = ctx->ws_vis;
   if (packed) p.ds = ctx->ws_ds;
   if (mode == IRGL_PERSISTENT && k == IRGL_SSSP && packed && !far && !use_local &&
@@ -888,12 +924,10 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
       if (stats) *stats = local;
       return IRGL_OK;
     }
-    DevStatus st;
-    s = read_status(ctx, &st);
+    s = wait_launch(ctx);
     local.rounds = ctx->st_host->rounds;
     local.last_out = ctx->st_host->last_out;
     local.edges_scanned = ctx->st_host->edges;
-    if (s == IRGL_OK) cudaMemsetAsync(&ctx->st->edges, 0, sizeof(unsigned long long), ctx->stream);
     if (stats) *stats = local;
     return s;
   }
@@ -915,15 +949,10 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
       if (stats) *stats = local;
       return IRGL_OK;
     }
-    DevStatus st;
-    s = read_status(ctx, &st);
+    s = wait_launch(ctx);
     local.rounds = ctx->st_host->rounds;
     local.last_out = ctx->st_host->last_out;
     local.edges_scanned = ctx->st_host->edges;
-    if (s == IRGL_OK) {
-      // edges accumulate across calls: clear for the next one
-      cudaMemsetAsync(&ctx->st->edges, 0, sizeof(unsigned long long), ctx->stream);
-    }
     if (stats) *stats = local;
     return s;
   }
@@ -997,12 +1026,12 @@ extern "C" {
 
 irgl_status irgl_iterate(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_worklist* initial, uint32_t* state_dev,
                          irgl_mode mode, const irgl_tuning* t, uint32_t max_rounds, irgl_stats* stats) {
-  return iterate_impl(ctx, k, g, initial, state_dev, mode, t, max_rounds, stats, true);
+  return iterate_impl(ctx, k, g, initial, state_dev, mode, t, max_rounds, stats, true, true);
 }
 
 irgl_status irgl_iterate_async(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_worklist* initial,
                                uint32_t* state_dev, const irgl_tuning* t, uint32_t max_rounds) {
-  return iterate_impl(ctx, k, g, initial, state_dev, IRGL_PERSISTENT, t, max_rounds, nullptr, false);
+  return iterate_impl(ctx, k, g, initial, state_dev, IRGL_PERSISTENT, t, max_rounds, nullptr, false, false);
 }
 
 irgl_status irgl_ctx_sync(irgl_ctx* ctx, irgl_stats* stats) {
@@ -1028,7 +1057,11 @@ irgl_status irgl_run(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, const uint32_t
   for (uint32_t i = 0; i < nsrc; ++i)
     if (srcs_host[i] >= g->n) return fail(IRGL_ERR_INVALID_ARG, "source %u out of range", srcs_host[i]);
   irgl_worklist* init = nullptr;
-  if (nsrc > 0 && nsrc <= kRunSrcMax) {
+  uint32_t inline_n = 0;
+  if (mode == IRGL_PERSISTENT && (k == IRGL_BFS || k == IRGL_SSSP) && nsrc > 0 && nsrc <= std::min(kInlineSrc, g->n) &&
+      !ctx->dbg_cap) {
+    inline_n = nsrc;  // a few sources travel in the kernel's parameters (no copy before the launch)
+  } else if (nsrc > 0 && nsrc <= kRunSrcMax) {
     // count and sources in one copy (no clear, push kernel or staging copy)
     if (!ctx->run_src) {
       cudaError_t e = cudaMalloc(&ctx->run_src, sizeof(uint32_t) * kRunSrcWords);
@@ -1076,24 +1109,23 @@ irgl_status irgl_run(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, const uint32_t
     }
     dst = ctx->ws_state;
   }
-  irgl_status s = iterate_impl(ctx, k, g, init, dst, mode, t, max_rounds, stats, !state_on_host);
+  ctx->isrc_n = inline_n;
+  if (inline_n) std::memcpy(ctx->isrc, srcs_host, sizeof(uint32_t) * inline_n);
+  irgl_status s = iterate_impl(ctx, k, g, init, dst, mode, t, max_rounds, stats, !state_on_host, true);
+  ctx->isrc_n = 0;
   if (s != IRGL_OK) return s;
   if (state_on_host) {
     cudaError_t e = cudaMemcpyAsync(state, dst, sizeof(uint32_t) * (size_t)g->n, cudaMemcpyDeviceToHost, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(e, "result copy");
     if (mode == IRGL_PERSISTENT) {
       // one wait for the launch, the result copy and the status read
-      DevStatus st;
-      s = read_status(ctx, &st);
+      s = wait_launch(ctx);
       if (stats) {
         stats->rounds = ctx->st_host->rounds;
         stats->last_out = ctx->st_host->last_out;
         stats->edges_scanned = ctx->st_host->edges;
       }
-      if (s != IRGL_OK) return s;
-      // cleared for the next call; later work on the stream runs after it
-      cudaMemsetAsync(&ctx->st->edges, 0, sizeof(unsigned long long), ctx->stream);
-      return IRGL_OK;
+      return s;
     }
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(e, "result copy");

@@ -153,6 +153,17 @@ struct Tune {
 };
 constexpr uint32_t kThreadBin = 4;
 
+// Outcome of a launch that the host waits for, written to pinned host memory by its
+// last CTA: with the record in place the stream's wait is all the host needs (no copy
+// of the status block back, no clear of the edge counter behind it). `seq` is written
+// last; a launch that ended early leaves it, and the host reads the status block.
+struct HostRec {
+  unsigned long long edges;
+  uint32_t err, rounds, last_out, epoch;
+  uint32_t seq;
+};
+constexpr uint32_t kInlineSrc = 8;  // sources that fit the kernel parameters
+
 // Single-graph kernel parameters.
 struct KParams {
   const uint32_t* __restrict__ row_ptr;
@@ -215,7 +226,26 @@ struct KParams {
   // is pushed again instead of expanded (defer_deg 0: off)
   uint32_t defer_deg;
   uint32_t defer_delta;
+  // BFS and SSSP: the initial items in the parameters themselves (isrc_n = 0: init_items)
+  uint32_t isrc_n;
+  uint32_t isrc[kInlineSrc];
+  HostRec* rec;      // nullptr: the host reads the status block
+  uint32_t rec_seq;
 };
+
+// Publish a launch's outcome (the thread that restores the status block, after it did).
+__device__ __forceinline__ void write_rec(DevStatus* st, HostRec* rec, uint32_t seq, uint32_t rounds, uint32_t last_out,
+                                          uint32_t epoch) {
+  const uint32_t err = __ldcg(&st->err);
+  rec->err = err;
+  rec->rounds = rounds;
+  rec->last_out = last_out;
+  rec->epoch = epoch;
+  // edges accumulate over the launches since the last one the host waited for
+  rec->edges = err == DERR_NONE ? atomicExch(&st->edges, 0ull) : 0ull;
+  __threadfence_system();
+  *reinterpret_cast<volatile uint32_t*>(&rec->seq) = seq;
+}
 
 // Per-launch (one round) arguments.
 struct RoundArgs {
@@ -2475,7 +2505,8 @@ template <int CTA>
 __device__ __forceinline__ void persistent_exit(Smem<CTA>& sm, DevStatus* st, bool ok, uint32_t rounds,
                                                 uint32_t last_out, uint32_t ep0, unsigned long long esum,
                                                 uint32_t* cont, uint32_t cont_buf, uint32_t far_buf = 0,
-                                                uint32_t far_n = 0, uint32_t id_step = 1) {
+                                                uint32_t far_n = 0, uint32_t id_step = 1, HostRec* rec = nullptr,
+                                                uint32_t rec_seq = 0) {
   __syncthreads();
   if (threadIdx.x == 0) {
     atomicAdd(&st->edges, esum);
@@ -2516,6 +2547,7 @@ __device__ __forceinline__ void persistent_exit(Smem<CTA>& sm, DevStatus* st, bo
     st->bu_n[0] = st->bu_n[1] = st->bu_n[2] = 0;
     st->pmin[0] = st->pmin[1] = st->pmin[2] = 0;
     st->exit_count = 0;
+    if (rec != nullptr) write_rec(st, rec, rec_seq, rounds, last_out, ep0 + rounds * id_step);
   }
   __threadfence();
 }
@@ -2579,7 +2611,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   DevStatus* st = p.st;
   uint32_t gen = 0;
   const uint32_t ep0 = __ldcg(&st->epoch);
-  const uint32_t init_n = p.init_count ? min(__ldcg(p.init_count), p.init_cap) : p.n;
+  const uint32_t init_n = p.isrc_n ? p.isrc_n : p.init_count ? min(__ldcg(p.init_count), p.init_cap) : p.n;
   if (p.skip_cta == static_cast<int>(blockIdx.x)) return;  // test hook: never arrives
 
   SingleView<OP> g{p.row_ptr, p.col, p.w, p.state, p.stamp, p.n};
@@ -2599,10 +2631,17 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   if (p.init_state) {
     uint32_t srcs[8];
     uint32_t ns = 0;
-    const bool small = base_op(OP) != OP_CC && p.init_items != nullptr && init_n <= 8;
+    const bool small = base_op(OP) != OP_CC && (p.isrc_n != 0 || p.init_items != nullptr) && init_n <= 8;
 #pragma unroll
-    for (uint32_t i = 0; i < 8; ++i) srcs[i] = (small && i < init_n) ? __ldcg(p.init_items + i) : kInf;
+    for (uint32_t i = 0; i < 8; ++i)
+      srcs[i] = (small && i < init_n) ? (p.isrc_n ? p.isrc[i] : __ldcg(p.init_items + i)) : kInf;
     if (small) ns = init_n;
+    if (base_op(OP) != OP_CC && p.isrc_n != 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+      // round 0's in-worklist (published by the prologue's barrier)
+#pragma unroll
+      for (uint32_t i = 0; i < 8; ++i)
+        if (i < ns) __stcg(p.items[0] + i, srcs[i]);
+    }
     if ((base_op(OP) == OP_SSSP || OP == OP_BFSR) && p.ds != nullptr) fill_packed(p.ds, p.n, srcs, ns, blockIdx.x * CTA + threadIdx.x, gridDim.x * CTA);
     else fill_state<OP>(p.state, p.n, srcs, ns, blockIdx.x * CTA + threadIdx.x, gridDim.x * CTA);
     if constexpr (OP == OP_BFS) {
@@ -2749,7 +2788,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
     uint32_t* const nxt = (r & 1) ? p.items[0] : p.items[1];
     RoundCtx rc;
     rc.in_n = in_n;
-    rc.in_items = r == 0 ? p.init_items : cur;
+    rc.in_items = r == 0 && (base_op(OP) == OP_CC || p.isrc_n == 0) ? p.init_items : cur;
     rc.out = Out{nxt, &st->tail[(r + 1) % 3], p.cap, &st->err};
     rc.bfs_val = r + 1;
     rc.ep = ep0 + r;
@@ -2926,7 +2965,7 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
   }
   const unsigned long long esum = cta_sum_u64<CTA>(sm, edges);
   trace_end(p.trace, p.trace_cap, rounds);
-  persistent_exit<CTA>(sm, st, ok, rounds, last_out, ep0, esum, nullptr, 0);
+  persistent_exit<CTA>(sm, st, ok, rounds, last_out, ep0, esum, nullptr, 0, 0, 0, 1, p.rec, p.rec_seq);
 }
 
 // Connected components by hooking and pointer jumping, in one cooperative
@@ -3162,7 +3201,7 @@ __device__ __forceinline__ void cc_jump_persistent(const KParams& p, Smem<kUfCta
   }
   const unsigned long long esum = cta_sum_u64<CTA>(sm, edges);
   trace_end(p.trace, p.trace_cap, rounds);
-  persistent_exit<CTA>(sm, st, ok, rounds, 0, ep0, esum, nullptr, 0);
+  persistent_exit<CTA>(sm, st, ok, rounds, 0, ep0, esum, nullptr, 0, 0, 0, 1, p.rec, p.rec_seq);
 }
 
 // One invocation (Invoke, or one round of a per-launch Iterate).

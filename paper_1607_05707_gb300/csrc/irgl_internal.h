@@ -20,6 +20,10 @@ struct irgl_ctx {
   int smem_optin = 0;  // opt-in shared memory per block (bytes)
   irgl::DevStatus* st = nullptr;       // device status block
   irgl::DevStatus* st_host = nullptr;  // pinned mirror
+  irgl::HostRec* rec = nullptr;      // pinned: outcome of the launch being waited for
+  uint32_t rec_seq = 0;              //   and its number
+  uint32_t isrc_n = 0;               // irgl_run: sources passed in the kernel parameters
+  uint32_t isrc[irgl::kInlineSrc] = {};
   uint32_t* run_src = nullptr;       // irgl_run sources (kRunSrcWords words, device)
   uint32_t* run_src_host = nullptr;  //   and their pinned mirror
   irgl_worklist* run_src_wl = nullptr;  // worklist view of run_src (owns nothing)
@@ -106,6 +110,7 @@ constexpr unsigned long long kRunTimeLimitNs = 60ull * 1000000000ull;  // persis
 unsigned long long run_time_limit_ns(const irgl_ctx* ctx);
 irgl_status resolve_tuning(const irgl_tuning* in, irgl_tuning* out);
 irgl_status read_status(irgl_ctx* ctx, DevStatus* out);
+irgl_status wait_launch(irgl_ctx* ctx);
 irgl_status status_from_device(const DevStatus& s);
 irgl_status control_cta(const uint32_t* masks, uint32_t count, uint32_t preferred, uint32_t* out);
 void reset_status(irgl_ctx* ctx);
@@ -125,4 +130,5 @@ irgl_status tune_descend(const std::function<float(const irgl_tuning&)>& measure
 }  // namespace irgl
 
 irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_worklist* initial, uint32_t* state_dev,
-                         irgl_mode mode, const irgl_tuning* tin, uint32_t max_rounds, irgl_stats* stats, bool sync);
+                         irgl_mode mode, const irgl_tuning* tin, uint32_t max_rounds, irgl_stats* stats, bool sync,
+                         bool record);

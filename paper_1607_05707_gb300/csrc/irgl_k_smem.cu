@@ -96,13 +96,18 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
   }
   __syncthreads();
   // round-0 worklist: the caller's initial items (CC without them: every vertex)
-  const uint32_t init_n = p.init_count ? min(__ldcg(p.init_count), p.init_cap) : n;
+  const uint32_t init_n = p.isrc_n ? p.isrc_n : p.init_count ? min(__ldcg(p.init_count), p.init_cap) : n;
   for (uint32_t base = 0; base < init_n; base += kSmemCta) {
     const uint32_t i = base + tid;
     bool push = false;
     uint32_t s = 0;
     if (i < init_n) {
-      s = p.init_items ? __ldcg(p.init_items + i) : i;
+      if (p.isrc_n) {
+#pragma unroll
+        for (uint32_t k = 0; k < kInlineSrc; ++k) s = i == k ? p.isrc[k] : s;
+      } else {
+        s = p.init_items ? __ldcg(p.init_items + i) : i;
+      }
       // a repeated source or item is pushed once (CC: a mark no round id reaches, rounds stay below n)
       if (s >= n) atomicCAS(&s_err, DERR_NONE, DERR_BAD_ITEM);
       else push = OP == OP_CC ? atomicExch(stamp + s, kInitMark) != kInitMark : atomicExch(val + s, 0u) != 0u;
@@ -211,6 +216,7 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
     st->rounds = rounds;
     st->last_out = last_out;
     if (s_err != DERR_NONE) atomicCAS(&st->err, DERR_NONE, s_err);
+    if (p.rec != nullptr) write_rec(st, p.rec, p.rec_seq, rounds, last_out, __ldcg(&st->epoch));
   }
 }
 

@@ -130,7 +130,7 @@ irgl_status irgl_autotune(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, const uin
     std::vector<float> ms;
     for (uint32_t r = 0; r <= reps; ++r) {  // first run warms up
       cudaEventRecord(e0, ctx->stream);
-      if (iterate_impl(ctx, k, g, init, ctx->ws_state, IRGL_PERSISTENT, &t, 0, nullptr, false) != IRGL_OK)
+      if (iterate_impl(ctx, k, g, init, ctx->ws_state, IRGL_PERSISTENT, &t, 0, nullptr, false, false) != IRGL_OK)
         return -1.f;
       cudaEventRecord(e1, ctx->stream);
       if (read_status(ctx, nullptr) != IRGL_OK) return -1.f;
