@@ -34,8 +34,10 @@
 // lock and fields (six arrays before). The lists (vertices, components, retries,
 // edges) are staged in shared memory and appended by one atomic per few hundred
 // items: one atomic per component on single counters was a third of the time
-// (2048^2 mesh, retry locks: link of the first iteration 2.03 ms of 6.4; now 2.0 ms in
-// all; blocking and ticket locks 14.7 and 13.0 -> 1.97 and 1.93 ms).
+// (2048^2 mesh, retry locks: link of the first iteration 2.03 ms of 6.4; 2.0 ms in
+// all with these, blocking and ticket locks 14.7 and 13.0 -> 1.97 and 1.93 ms; then 1.65
+// ms with the first iteration apart, where every vertex is its own component: no
+// component reads, no contention for a record).
 //
 // Outlined (IRGL_PERSISTENT): the three kernels run back to back in one
 // cooperative launch, separated by the grid barrier; the CTA size is chosen by
@@ -128,8 +130,9 @@ struct MinEdge {
 __device__ __forceinline__ MinEdge no_edge() { return MinEdge{kInf, kInf, kInf, 0u, 0u}; }
 
 // Lightest cross-component edge among u's edges [beg, end), lanes taking
-// every stride-th edge from beg + rank, four columns, components and weights in
-// flight.
+// every stride-th edge from beg + rank, four columns, then their components and
+// weights in flight. FIRST: the first iteration, every vertex its own component.
+template <bool FIRST>
 __device__ __forceinline__ void scan_edges(const MsfParams& p, uint32_t u, uint32_t cu, uint32_t beg, uint32_t end,
                                            uint32_t rank, uint32_t stride, MinEdge& best) {
   for (unsigned long long e0 = static_cast<unsigned long long>(beg) + rank; e0 < end; e0 += 4ull * stride) {
@@ -137,9 +140,10 @@ __device__ __forceinline__ void scan_edges(const MsfParams& p, uint32_t u, uint3
 #pragma unroll
     for (uint32_t k = 0; k < 4; ++k) v[k] = e0 + k * stride < end ? __ldg(p.col + e0 + k * stride) : u;
 #pragma unroll
-    for (uint32_t k = 0; k < 4; ++k) cv[k] = v[k] != u ? __ldcg(p.comp + v[k]) : cu;
-#pragma unroll
-    for (uint32_t k = 0; k < 4; ++k) wt[k] = cv[k] != cu ? static_cast<uint32_t>(__ldg(p.w + e0 + k * stride)) : kInf;
+    for (uint32_t k = 0; k < 4; ++k) {
+      cv[k] = FIRST ? v[k] : v[k] != u ? __ldcg(p.comp + v[k]) : cu;
+      wt[k] = e0 + k * stride < end ? static_cast<uint32_t>(__ldg(p.w + e0 + k * stride)) : kInf;
+    }
 #pragma unroll
     for (uint32_t k = 0; k < 4; ++k) {
       if (cv[k] == cu) continue;
@@ -301,12 +305,25 @@ __device__ __forceinline__ bool aggregate_update(const MsfParams& p, bool found,
   return !atomic_update(p, cu, best, first, locks);
 }
 
-// find_min over a worklist: `in` (nullptr = vertices 0..in_n-1). Default
+// The Atomic section of a component of one vertex, in the first iteration: no other
+// thread touches its record, so the lock (free unless the test hook holds it) need not
+// be taken and the record is two plain stores.
+__device__ __forceinline__ bool first_update(const MsfParams& p, uint32_t u, const MinEdge& k, bool& first, uint32_t& locks) {
+  if (u == p.held_lock) return atomic_update(p, u, k, first, locks);
+  MsfRec* const r = p.rec + u;
+  __stcg(reinterpret_cast<ulonglong2*>(r), make_ulonglong2(wl_of(k), wl_of(k)));
+  __stcg(reinterpret_cast<uint4*>(&r->hi), make_uint4(k.hi, k.e, k.other, 0u));
+  first = true;
+  ++locks;
+  return true;
+}
+
+// find_min over a worklist: `in` (nullptr = vertices 0..in_n-1, in the first iteration). Default
 // mapping: a warp takes 32 consecutive items; lists of 32 edges or more are
 // scanned by the whole warp. Retry mapping (Retry Backoff): thread t takes the
 // contiguous block [t * B, (t + 1) * B) and scans each list alone. Trip counts
 // are CTA-uniform (the lists are flushed by the whole CTA).
-template <int CTA>
+template <int CTA, bool FIRST>
 __device__ void msf_find_min(const MsfParams& p, Smem<CTA>& sm, MsfLists<CTA>& ls, const uint32_t* in, uint32_t in_n,
                              bool backoff, uint32_t* out, uint32_t out_base, uint32_t* retry_out, MsfSlot* slot,
                              uint32_t comp_base) {
@@ -324,25 +341,27 @@ __device__ void msf_find_min(const MsfParams& p, Smem<CTA>& sm, MsfLists<CTA>& l
     const bool valid = idx < in_n;
     uint32_t u = 0, cu = 0, beg = 0, end = 0;
     if (valid) {
-      u = in ? __ldcg(in + idx) : static_cast<uint32_t>(idx);
-      cu = __ldcg(p.comp + u);
+      u = FIRST ? static_cast<uint32_t>(idx) : __ldcg(in + idx);
+      cu = FIRST ? u : __ldcg(p.comp + u);
       beg = __ldg(p.row_ptr + u);
       end = __ldg(p.row_ptr + u + 1);
     }
     MinEdge best = no_edge();
     const bool big = !backoff && valid && end - beg >= 32u;
-    if (valid && !big) scan_edges(p, u, cu, beg, end, 0, 1, best);
+    if (valid && !big) scan_edges<FIRST>(p, u, cu, beg, end, 0, 1, best);
     for (unsigned m = __ballot_sync(kFull, big); m; m &= m - 1) {
       const int l = __ffs(m) - 1;
       MinEdge wb = no_edge();
-      scan_edges(p, __shfl_sync(kFull, u, l), __shfl_sync(kFull, cu, l), __shfl_sync(kFull, beg, l),
+      scan_edges<FIRST>(p, __shfl_sync(kFull, u, l), __shfl_sync(kFull, cu, l), __shfl_sync(kFull, beg, l),
                  __shfl_sync(kFull, end, l), lane, 32, wb);
       wb = warp_min_edge(wb);
       if (lane == static_cast<uint32_t>(l)) best = wb;
     }
     const bool found = best.w != kInf;
     bool first = false;
-    const bool missed = aggregate_update(p, found, cu, best, first, locks);
+    bool missed;
+    if (FIRST) missed = found && !first_update(p, u, best, first, locks);
+    else missed = aggregate_update(p, found, cu, best, first, locks);
     __syncwarp();
     stage_item<CTA>(sm, ls, 0, found && !missed, u);
     stage_item<CTA>(sm, ls, 1, first, cu);
@@ -500,7 +519,10 @@ __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_msf(MsfParams p)
     const unsigned long long t_retry0 = msf_now();
     for (;;) {
       begin_invocation();
-      msf_find_min<CTA>(p, sm, ls, fin, fin_n, backoff, out, out_total, p.retry[rb], &ms->slot[inv % 3], comp_total);
+      if (fin == nullptr)
+        msf_find_min<CTA, true>(p, sm, ls, fin, fin_n, false, out, out_total, p.retry[rb], &ms->slot[inv % 3], comp_total);
+      else
+        msf_find_min<CTA, false>(p, sm, ls, fin, fin_n, backoff, out, out_total, p.retry[rb], &ms->slot[inv % 3], comp_total);
       const MsfSlot s = end_invocation();
       if (!ok) break;
       out_total += s.out;
@@ -568,8 +590,11 @@ __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_msf_step(MsfPara
     case MSF_INIT: msf_init(p, gtid, nthreads); break;
     case MSF_FIND:
     case MSF_FIND_RETRY:
-      msf_find_min<CTA>(p, sm, ls, s.in, s.in_n, s.phase == MSF_FIND_RETRY, s.out, s.out_base, s.retry_out, slot,
-                        s.comp_base);
+      if (s.in == nullptr)
+        msf_find_min<CTA, true>(p, sm, ls, s.in, s.in_n, false, s.out, s.out_base, s.retry_out, slot, s.comp_base);
+      else
+        msf_find_min<CTA, false>(p, sm, ls, s.in, s.in_n, s.phase == MSF_FIND_RETRY, s.out, s.out_base, s.retry_out, slot,
+                                 s.comp_base);
       break;
     case MSF_LINK: msf_link<CTA>(p, sm, ls, s.comp_n); break;
     case MSF_JUMP: {
