@@ -18,8 +18,8 @@
 // list counters in turn), a warp's pushes one atomic, and a frontier of up to 256
 // items gives every item four lanes, dealt across the warps; larger ones have their
 // edges dealt to the lanes by a scan. 64 x 64 grid BFS, 113 rounds: 1.1 us a round
-// and 128 us a call before, 0.65 and 99.5 us now; R-MAT of 2^10 vertices, SSSP: 97
-// -> 62 us (rounds of 360-525 items 5-10 us before, and 13 us went to 1024 threads
+// and 128 us a call before, 0.65 and 99.5 us with these (narrow rounds below); R-MAT of
+// 2^10 vertices, SSSP: 97 -> 62 us (rounds of 360-525 items 5-10 us before, and 13 us went to 1024 threads
 // adding their edge counts to one 64-bit word).
 //
 // Shared-memory layout (32-bit words): row_ptr[n + 1], col[m], w[m] (SSSP),
@@ -36,6 +36,22 @@ namespace {
 constexpr int kSmemCta = 1024;
 constexpr uint32_t kSmemWarps = kSmemCta / 32;
 constexpr uint32_t kSmemFour = kSmemCta / 4;  // frontiers of at most this many items give each four lanes
+// Narrow rounds: a frontier of at most 64 items is one pass of eight warps, which cross a
+// barrier of their own faster than 32 warps cross the CTA's; the others wait at the next
+// CTA barrier until a frontier outgrows them (64 x 64 grid BFS 104 -> 87
+// us a call, SSSP on a 20 x 24 mesh 51 -> 42; 256 threads for the whole run instead
+// slow down wider frontiers: SSSP on a 50 x 60 mesh 89 -> 110).
+constexpr uint32_t kNarrowWarps = 8;
+constexpr uint32_t kNarrow = kNarrowWarps * 8;
+
+// Barrier of the first kNarrowWarps warps with the or of `p`.
+__device__ __forceinline__ int narrow_sync_or(int p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred a, b;\n\tsetp.ne.s32 a, %1, 0;\n\tbarrier.cta.red.or.pred b, 1, %2, a;\n\tselp.s32 %0, 1, 0, b;\n\t}"
+      : "=r"(r) : "r"(p), "n"(kNarrowWarps * 32) : "memory");
+  return r;
+}
 constexpr uint32_t kInitMark = 0xFFFFFFFEu;  // stamp of the round-0 items (CC)
 
 // Warp-aggregated push: one shared atomic per warp that pushes anything.
@@ -62,11 +78,50 @@ __device__ __forceinline__ bool smem_relax(const uint32_t* w, uint32_t* val_arr,
   return nd < val_arr[v] && nd < atomicMin(val_arr + v, nd) && atomicExch(stamp + v, r) != r;
 }
 
+// A round over at most 8 * warps items by `warps` warps: four lanes per item, items
+// dealt across the warps, so a short list is one step of one warp without a search
+// for an edge's owner. Returns the edges of the lists this lane leads.
+template <uint32_t OP>
+__device__ __forceinline__ uint32_t smem_four(const uint32_t* in, uint32_t in_n, uint32_t warps, const uint32_t* rp,
+                                              const uint32_t* col, const uint32_t* w, uint32_t* val, uint32_t* stamp,
+                                              uint32_t r, uint32_t* out, uint32_t* out_n, uint32_t n, uint32_t* err) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 3;
+  if (warp >= in_n) return 0u;
+  const uint32_t i = (lane >> 2) * warps + warp;
+  uint32_t b = 0, e = 0, x = 0;
+  if (i < in_n) {
+    const uint32_t u = in[i];
+    b = rp[u];
+    e = rp[u + 1];
+    x = OP == OP_BFS ? r + 1u : val[u];
+  }
+  const bool lng = e - b > 32u;
+  const uint32_t trips = __reduce_max_sync(kFull, lng ? 0u : (e - b + 3u) >> 2);
+  for (uint32_t t = 0; t < trips; ++t) {
+    const uint32_t k = b + 4u * t + sub;
+    const bool mine = !lng && k < e;
+    const uint32_t v = mine ? col[k] : 0u;
+    smem_push(out, out_n, n, mine && smem_relax<OP>(w, val, stamp, k, v, x, r), v, err);
+  }
+  for (unsigned mk = __ballot_sync(kFull, lng && sub == 0); mk; mk &= mk - 1) {
+    const int ld = __ffs(mk) - 1;
+    const uint32_t lb = __shfl_sync(kFull, b, ld), le = __shfl_sync(kFull, e, ld);
+    const uint32_t lx = __shfl_sync(kFull, x, ld);
+    for (uint32_t k0 = lb; k0 < le; k0 += 32) {
+      const uint32_t k = k0 + lane;
+      const uint32_t v = k < le ? col[k] : 0u;
+      smem_push(out, out_n, n, k < le && smem_relax<OP>(w, val, stamp, k, v, lx, r), v, err);
+    }
+  }
+  return sub == 0 ? e - b : 0u;
+}
+
 template <uint32_t OP>
 __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
   extern __shared__ __align__(16) uint32_t sh[];
   __shared__ uint32_t s_n[3];  // worklist sizes by round mod 3
   __shared__ uint32_t s_err;
+  __shared__ uint32_t s_round, s_done;  // where the narrow rounds ended
   __shared__ unsigned long long s_edges;
   const unsigned long long t_start = p.trace ? globaltimer_ns() : 0ull;
   const uint32_t tid = threadIdx.x, lane = tid & 31;
@@ -118,45 +173,48 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
   trace_prologue(p.trace, p.trace_cap, t_start, s_n[0]);
   const uint32_t warp = tid >> 5;
   uint32_t edges = 0, rounds = 0, last_out = 0;
-  for (uint32_t r = 0;; ++r) {
+  bool done = false;
+  for (uint32_t r = 0; !done; ++r) {
+    const uint32_t in_n = min(s_n[r % 3], n);  // a worklist holds at most n items
+    if (in_n <= kNarrow) {
+      // narrow rounds, until the frontier outgrows them or the run ends; every thread
+      // has read the sizes of the rounds before when they start to reuse the counters
+      __syncthreads();
+      if (warp < kNarrowWarps) {
+        for (uint32_t now = in_n;; ++r) {
+          uint32_t* const out_n = &s_n[(r + 1) % 3];
+          if (tid == 0) s_n[(r + 2) % 3] = 0;
+          edges += smem_four<OP>((r & 1) ? wl1 : wl0, now, kNarrowWarps, rp, col, w, val, stamp, r, (r & 1) ? wl0 : wl1,
+                                 out_n, n, &s_err);
+          const int bad = narrow_sync_or(*reinterpret_cast<volatile uint32_t*>(&s_err) != DERR_NONE);
+          last_out = min(*reinterpret_cast<volatile uint32_t*>(out_n), n);
+          rounds = r + 1;
+          trace_round(p.trace, p.trace_cap, rounds, now, last_out);
+          done = last_out == 0 || bad;
+          if (!done && rounds >= p.max_rounds) {
+            if (tid == 0) atomicCAS(&s_err, DERR_NONE, DERR_MAX_ROUNDS);
+            done = true;
+          }
+          if (done || last_out > kNarrow) break;
+          now = last_out;
+        }
+        if (tid == 0) {
+          s_round = r;
+          s_done = done;
+        }
+      }
+      __syncthreads();
+      r = s_round;  // the last round that ran
+      done = s_done != 0;
+      continue;
+    }
     uint32_t* in = (r & 1) ? wl1 : wl0;
     uint32_t* out = (r & 1) ? wl0 : wl1;
     uint32_t* out_n = &s_n[(r + 1) % 3];
-    const uint32_t in_n = min(s_n[r % 3], n);  // a worklist holds at most n items
     // the counter of round r + 1's pushes: last read at the start of round r - 1, before its barrier
     if (tid == 0) s_n[(r + 2) % 3] = 0;
     if (in_n <= kSmemFour) {
-      // Four lanes per item, items dealt across the warps: a short list is one
-      // step of one warp, no search for an edge's owner
-      const uint32_t i = (lane >> 2) * kSmemWarps + warp, sub = lane & 3;
-      if (warp < in_n) {
-        uint32_t b = 0, e = 0, x = 0;
-        if (i < in_n) {
-          const uint32_t u = in[i];
-          b = rp[u];
-          e = rp[u + 1];
-          x = OP == OP_BFS ? r + 1u : val[u];
-        }
-        if (sub == 0) edges += e - b;
-        const bool lng = e - b > 32u;
-        const uint32_t trips = __reduce_max_sync(kFull, lng ? 0u : (e - b + 3u) >> 2);
-        for (uint32_t t = 0; t < trips; ++t) {
-          const uint32_t k = b + 4u * t + sub;
-          const bool mine = !lng && k < e;
-          const uint32_t v = mine ? col[k] : 0u;
-          smem_push(out, out_n, n, mine && smem_relax<OP>(w, val, stamp, k, v, x, r), v, &s_err);
-        }
-        for (unsigned mk = __ballot_sync(kFull, lng && sub == 0); mk; mk &= mk - 1) {
-          const int ld = __ffs(mk) - 1;
-          const uint32_t lb = __shfl_sync(kFull, b, ld), le = __shfl_sync(kFull, e, ld);
-          const uint32_t lx = __shfl_sync(kFull, x, ld);
-          for (uint32_t k0 = lb; k0 < le; k0 += 32) {
-            const uint32_t k = k0 + lane;
-            const uint32_t v = k < le ? col[k] : 0u;
-            smem_push(out, out_n, n, k < le && smem_relax<OP>(w, val, stamp, k, v, lx, r), v, &s_err);
-          }
-        }
-      }
+      edges += smem_four<OP>(in, in_n, kSmemWarps, rp, col, w, val, stamp, r, out, out_n, n, &s_err);
     } else {
       // The warp's items (dealt across the warps) have their edges dealt out to
       // its lanes, two per lane and step, owners by a shuffle search
@@ -198,10 +256,10 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
     last_out = min(*out_n, n);
     rounds = r + 1;
     trace_round(p.trace, p.trace_cap, rounds, in_n, last_out);
-    if (last_out == 0 || bad) break;
-    if (rounds >= p.max_rounds) {
+    done = last_out == 0 || bad;
+    if (!done && rounds >= p.max_rounds) {
       if (tid == 0) atomicCAS(&s_err, DERR_NONE, DERR_MAX_ROUNDS);
-      break;
+      done = true;
     }
   }
   for (uint32_t v = tid; v < n; v += kSmemCta) __stcg(p.state + v, val[v]);
