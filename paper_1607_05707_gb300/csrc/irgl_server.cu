@@ -851,7 +851,8 @@ irgl_status irgl_server_create(irgl_ctx* ctx, const irgl_server_config* cfg, irg
   }
   DevStatus z;
   std::memset(&z, 0, sizeof(z));
-  z.epoch = 1;
+  // admission stamps "last pushed one round ago", epoch - id_step: not below 0 in the first epoch
+  z.epoch = s->id_step;
   *s->st_host = z;
   e = cudaMemcpyAsync(s->st, s->st_host, sizeof(DevStatus), cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess && s->stamp) e = cudaMemsetAsync(s->stamp, 0, sizeof(uint32_t) * s->arena_n, s->stream);

@@ -82,3 +82,21 @@ def test_mixed_batches(ctx, delta, cta):
         b.close()
     for h in handles:
         h.close()
+
+
+@pytest.mark.parametrize("k", [0, 1, 15])
+def test_server_first_epoch_isolated_source(ctx, k):
+    # a query that never pushes, admitted in a server's first epoch
+    from paper_1607_05707_gb300.api import Server
+
+    g = inputs.csr_from_edges(50, [1, 2], [2, 3], [4, 5])
+    dg = ctx.load(g)
+    for kind in ("sssp", "bfs"):
+        srv = Server(ctx, arena_bytes=1 << 20, max_slots=4, epoch_rounds=8, tuning=dict(flags=k << 8), solo_min_n=0xFFFFFFFF)
+        out = np.zeros(50, np.uint32)
+        t = srv.submit(kind, dg, 7, out)
+        srv.drain(10.0)
+        assert srv.poll(t)["status"] == 0
+        np.testing.assert_array_equal(out, oracle.run(kind, g, np.array([7], np.uint32)))
+        srv.close()
+    dg.close()
