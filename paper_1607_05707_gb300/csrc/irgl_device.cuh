@@ -38,8 +38,9 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // since a vertex can be reached there before its level is final.
 // OP_SSSPF, OP_CCF: SSSP and min-label CC with the near-far schedule, kernels of
 // their own: its lists and limits kept in registers beside the plain rounds' code
-// made the plain SSSP kernel spill (112 bytes of spill loads, 20 without). OP_SSSPL, OP_SSSPFL: launch table entries of the
-// SSSP and near-far SSSP kernels with CTA-local sub-rounds (LOCAL below).
+// made the plain SSSP kernel spill (112 bytes of spill loads, 20 without).
+// OP_SSSPL, OP_SSSPFL: launch table entries of the SSSP and near-far SSSP kernels
+// with CTA-local sub-rounds (LOCAL below).
 enum : uint32_t { OP_BFS = 0, OP_SSSP = 1, OP_CC = 2, OP_RUNTIME = 3, OP_CCJ = 4, OP_BFSR = 5, OP_SSSPL = 6, OP_SSSPF = 7,
                   OP_CCF = 8, OP_SSSPFL = 9 };
 
