@@ -97,8 +97,12 @@ typedef struct {
                              the rounds below the limit drain; 0 = plain rounds (every improvement
                              is pushed). CC with delta = 1 floods the smallest label first, so
                              each vertex mostly takes its final label once. SSSP on a graph of short
-                             lists (m <= 6 n, none at the degree thresholds) takes CTA-local sub-rounds
-                             in its sparse rounds by itself (up to 16 worklist entries per vertex). Batches and servers:
+                             lists (m <= 6 n, none at the degree thresholds; lengths the host does not
+                             know count as short unless IRGL_TUNE_NO_SPLIT is set) takes 15 CTA-local
+                             sub-rounds in its sparse rounds by itself, with two worklists of their own:
+                             n entries each and 192 per CTA and edge of the longest short list (16 n at
+                             most). A device without room for them gets plain rounds, same distances.
+                             IRGL_TUNE_LOCAL is not read there. Batches and servers:
                              per-query near-far for their SSSP queries (below) */
   uint32_t defer_deg;     /* persistent SSSP with plain rounds (delta = 0, no sub-rounds): a popped
                              vertex with at least defer_deg out-edges whose distance is above the
@@ -124,7 +128,8 @@ typedef struct {
                                     Pays on high-diameter graphs (meshes, grids), costs extra work on
                                     low-diameter ones (R-MAT); irgl_autotune tries k = 0, 4, 15.
                                     max_rounds is capped at 2^32 / (k + 1) - 1 global rounds.
-                                    Ignored with IRGL_TUNE_DIROPT or IRGL_TUNE_NO_PACKED. */
+                                    Ignored with IRGL_TUNE_DIROPT or IRGL_TUNE_NO_PACKED, and by a
+                                    single SSSP query with delta != 0 (see there). */
 #define IRGL_TUNE_NO_PACKED 0x8u /* persistent SSSP: keep distances and the dedup stamps in two
                                     arrays (by default one 64-bit word per vertex holds both,
                                     lowered by one atomicMin, and the distances are copied to the
@@ -551,7 +556,9 @@ irgl_status irgl_msf(irgl_ctx* ctx, irgl_graph* g, irgl_mode mode, irgl_lock loc
  *   key 8: 1 = persistent Iterate, batch and server rounds whose frontier is
  *          smaller than one tile per CTA keep it in static per-CTA spans
  *          instead of spreading it over every CTA (batches and servers read it
- *          when they are prepared or run an epoch). */
+ *          when they are prepared or run an epoch).
+ *   key 9: 1 = the worklists of near-far sub-rounds are refused, as if the
+ *          device had no room for them. */
 irgl_status irgl_debug_set(irgl_ctx* ctx, int key, int64_t value);
 
 #ifdef __cplusplus

@@ -269,6 +269,41 @@ uint32_t persistent_grid(irgl_ctx* ctx, uint32_t op, const irgl_tuning& t) {
   return std::max<uint32_t>(grid, 1);
 }
 
+// Worklists of a near-far Iterate with sub-rounds (ctx->ws_near); false when the device
+// has no room for them. They are lists of their own, not ws_items grown: a refusal
+// leaves the call its plain rounds, and other calls keep the lists they have. Entries:
+// n for the pushes outside local_round (at most one per vertex and round) and, in
+// local_round, the pushes of a CTA's last sub-round only, over at most kNearGrow +
+// 2 * kNearLocal items of lists below the degree thresholds (longer ones go to the big
+// list). A first call on a 1021 x 1031 mesh of unknown degrees takes 115 MB of device
+// memory in all (203 with a list entry per vertex and sub-round). Not so many sub-rounds
+// on large graphs to save memory is slower: 3000 x 3000 mesh 23.7 ms with three, 17.3
+// with fifteen; 6000 x 6000 128 ms with none, 38.4 with fifteen.
+bool near_lists(irgl_ctx* ctx, const irgl_graph* g, const irgl_tuning& t) {
+  if (ctx->dbg_cap) return true;  // ws_items, of that capacity
+  const uint64_t longest = g->max_deg != 0xFFFFFFFFu ? g->max_deg : std::min(t.warp_thresh, t.cta_thresh) - 1u;
+  const uint64_t local = static_cast<uint64_t>(persistent_grid(ctx, OP_SSSPFL, t)) * (kNearGrow + 2u * kNearLocal) * longest;
+  const uint64_t want = std::max<uint64_t>(std::min<uint64_t>({g->n + local, 16ull * g->n, 0xFFFFFFF0ull}), 1);
+  if (want <= ctx->ws_near_cap) return true;
+  if (want >= ctx->ws_near_refused || ctx->dbg_no_near) return false;
+  cudaStreamSynchronize(ctx->stream);
+  cudaFree(ctx->ws_near[0]);
+  cudaFree(ctx->ws_near[1]);
+  ctx->ws_near[0] = ctx->ws_near[1] = nullptr;
+  ctx->ws_near_cap = 0;
+  cudaError_t e = cudaMalloc(&ctx->ws_near[0], sizeof(uint32_t) * static_cast<size_t>(want));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->ws_near[1], sizeof(uint32_t) * static_cast<size_t>(want));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // handled: no later launch check may find it
+    cudaFree(ctx->ws_near[0]);
+    ctx->ws_near[0] = nullptr;
+    ctx->ws_near_refused = want;  // asked once: a failing allocation costs a call more than the rounds save
+    return false;
+  }
+  ctx->ws_near_cap = static_cast<uint32_t>(want);
+  return true;
+}
+
 uint32_t op_of(irgl_kernel k) { return k == IRGL_CC_JUMP ? OP_CCJ : static_cast<uint32_t>(k); }
 
 irgl_status check_kernel_graph(irgl_kernel k, const irgl_graph* g) {
@@ -407,6 +442,8 @@ irgl_status irgl_ctx_destroy(irgl_ctx* ctx) {
   cudaFree(ctx->ws_far[0]);
   cudaFree(ctx->ws_far[1]);
   cudaFree(ctx->ws_far_stamp);
+  cudaFree(ctx->ws_near[0]);
+  cudaFree(ctx->ws_near[1]);
   cudaFree(ctx->ws_state);
   cudaFree(ctx->trace);
   cudaFree(ctx->big_e);
@@ -495,6 +532,7 @@ irgl_status irgl_debug_set(irgl_ctx* ctx, int key, int64_t value) {
     case 7: ctx->dbg_time_limit_ms = value > 0 ? static_cast<uint64_t>(value) : 0; return IRGL_OK;
     case 8: ctx->dbg_no_spread = value > 0 ? 1u : 0u; return IRGL_OK;
     case 5: ctx->dbg_force_bottom_up = value > 0 ? 1u : 0u; return IRGL_OK;
+    case 9: ctx->dbg_no_near = value > 0 ? 1u : 0u; return IRGL_OK;
     case 6: ctx->dbg_held_lock = value >= 0 ? static_cast<uint32_t>(value) : 0xFFFFFFFFu; return IRGL_OK;
   }
   return fail(IRGL_ERR_INVALID_ARG, "unknown debug key %d", key);
@@ -845,18 +883,23 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   const bool packed = (k == IRGL_SSSP || (k == IRGL_BFS && use_local)) && mode == IRGL_PERSISTENT &&
                       !(t.flags & IRGL_TUNE_NO_PACKED);
   const bool far = (k == IRGL_SSSP || k == IRGL_CC) && mode == IRGL_PERSISTENT && t.delta != 0;
+  const bool smem = mode == IRGL_PERSISTENT && !(t.flags & IRGL_TUNE_NO_SMEM) && k != IRGL_CC_JUMP &&
+                    ctx->smem_optin > static_cast<int>(kSmemStaticReserve) &&
+                    smem_iterate_fits(op_of(k), g->n, g->m, static_cast<size_t>(ctx->smem_optin) - kSmemStaticReserve);
   // Near-far SSSP on a graph of short lists takes sub-rounds in its sparse rounds by
   // itself: a frontier of a mesh or road network (m / n of 2 to 5) advances a hop per
   // round; one of a power-law graph reaches everything in a few dozen rounds and only
   // rescans (R-MAT of 2^18 vertices, 4 edges each: 298 us plain, 383 with sub-rounds), so
-  // a long list, known here or met on the device, turns them off. Fewer of them on
-  // larger graphs, whose worklists (n entries per sub-round id) would pass 0.5 GB each.
-  const bool short_lists = g->m <= 6ull * g->n && (g->max_deg == 0xFFFFFFFFu || g->max_deg < std::min(t.warp_thresh, t.cta_thresh));
-  const uint32_t near_rounds = !(far && packed && k == IRGL_SSSP && short_lists) ? 0u
-                               : g->n <= (1u << 23) ? 15u : g->n <= (1u << 25) ? 3u : 0u;
+  // a long list, known here or met on the device, turns them off. Without the big list a
+  // list of unknown length is met by nothing, so unknown degrees then turn them off too.
+  const bool known = g->max_deg != 0xFFFFFFFFu;
+  const bool short_lists = g->m <= 6ull * g->n && (known ? g->max_deg < std::min(t.warp_thresh, t.cta_thresh)
+                                                         : !(t.flags & IRGL_TUNE_NO_SPLIT));
+  uint32_t near_rounds = far && packed && k == IRGL_SSSP && short_lists && !smem ? 15u : 0u;
   // a vertex can be pushed once per sub-round: worklists of n * (sub-rounds + 1)
-  s = ensure_workspace(ctx, g->n, k != IRGL_BFS, far, vis, packed, (use_local ? sub_rounds : near_rounds) + 1u);
+  s = ensure_workspace(ctx, g->n, k != IRGL_BFS, far, vis, packed, use_local ? sub_rounds + 1u : 1u);
   if (s != IRGL_OK) return s;
+  if (near_rounds && !near_lists(ctx, g, t)) near_rounds = 0;  // no room for their lists: plain rounds
   const uint32_t op = use_local ? (k == IRGL_BFS ? OP_BFSR : OP_SSSPL)
                       : far ? (k == IRGL_SSSP ? (near_rounds ? OP_SSSPFL : OP_SSSPF) : OP_CCF) : op_of(k);
   if (k == IRGL_CC_JUMP) t.cta_size = kUfCta;  // its vertex blocks fill an SM's shared memory: one CTA each
@@ -901,6 +944,11 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   if (use_local || near_rounds) {
     p.local_rounds = use_local ? sub_rounds : near_rounds;
     p.diropt = 0;
+    if (near_rounds && !ctx->dbg_cap) {
+      p.items[0] = ctx->ws_near[0];
+      p.items[1] = ctx->ws_near[1];
+      p.cap = ctx->ws_near_cap;
+    }
     // round r stamps with ids r * (sub-rounds + 1) + 1 .. (r + 1) * (sub-rounds + 1):
     // stop before they would wrap to 0, the "on no worklist" stamp
     p.max_rounds = std::min(p.max_rounds, 0xFFFFFFFFu / (p.local_rounds + 1u) - 1u);
@@ -909,9 +957,7 @@ irgl_status iterate_impl(irgl_ctx* ctx, irgl_kernel k, irgl_graph* g, irgl_workl
   std::memset(&local, 0, sizeof(local));
   local.cta_size = t.cta_size;
 
-  if (mode == IRGL_PERSISTENT && !(t.flags & IRGL_TUNE_NO_SMEM) && k != IRGL_CC_JUMP &&
-      ctx->smem_optin > static_cast<int>(kSmemStaticReserve) &&
-      smem_iterate_fits(op_of(k), g->n, g->m, static_cast<size_t>(ctx->smem_optin) - kSmemStaticReserve)) {
+  if (smem) {
     // the whole Iterate in one CTA, the graph in shared memory (schedule choices
     // such as sub-rounds, near-far or bottom-up rounds do not apply to it)
     p.skip_cta = -1;

@@ -35,6 +35,9 @@ struct irgl_ctx {
   uint32_t* ws_far[2] = {nullptr, nullptr};  // SSSP near-far lists
   uint32_t* ws_far_stamp = nullptr;
   uint32_t ws_far_n = 0;
+  uint32_t* ws_near[2] = {nullptr, nullptr};  // worklists of a near-far Iterate with sub-rounds
+  uint32_t ws_near_cap = 0;
+  uint64_t ws_near_refused = ~0ull;           //   a capacity that the device had no room for
   uint32_t* ws_stamp = nullptr;  // SSSP/CC push dedup stamps
   uint32_t ws_stamp_n = 0;
   uint32_t* msf_buf = nullptr;   // minimum spanning forest workspace (status block + 16 arrays of msf_n)
@@ -55,6 +58,7 @@ struct irgl_ctx {
   // test hooks
   uint64_t dbg_timeout_us = 0;
   uint64_t dbg_time_limit_ms = 0;  // wall-time limit of persistent launches (0: the default)
+  uint32_t dbg_no_near = 0;        // 1: the lists of near-far sub-rounds are refused
   uint32_t dbg_no_spread = 0;      // 1: sub-grid frontiers stay in static per-CTA spans
   int dbg_skip_cta = -1;
   uint32_t dbg_cap = 0;
