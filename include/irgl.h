@@ -525,7 +525,8 @@ typedef struct {
   uint64_t weight;       /* sum of the forest edges' weights */
   uint32_t invocations;  /* kernel invocations inside the Pipe (find_min, retries, link, jump passes) */
   uint32_t retries;      /* vertices pushed to the retry worklist (IRGL_LOCK_RETRY) */
-  uint32_t locks;        /* lock acquisitions (the rest passed the pre-lock weight test) */
+  uint32_t locks;        /* lock acquisitions (the rest passed the pre-lock weight test; the first
+                            iteration, every vertex its own component, takes none) */
   uint32_t launches;     /* kernel launches */
   uint32_t grid;
   uint32_t cta_size;

@@ -314,7 +314,6 @@ __device__ __forceinline__ bool first_update(const MsfParams& p, uint32_t u, con
   __stcg(reinterpret_cast<ulonglong2*>(r), make_ulonglong2(wl_of(k), wl_of(k)));
   __stcg(reinterpret_cast<uint4*>(&r->hi), make_uint4(k.hi, k.e, k.other, 0u));
   first = true;
-  ++locks;
   return true;
 }
 

@@ -25,3 +25,19 @@ def test_chains_and_stages(ctx, n):  # noqa: F811
             check(ctx, g, dg, "persistent", lock, dict(cta_size=1024))
         check(ctx, g, dg, "per_launch", "retry", dict(cta_size=256))
         dg.close()
+
+
+@pytest.mark.parametrize("lock", ["blocking", "ticket", "retry"])
+@pytest.mark.parametrize("mode", ["persistent", "per_launch"])
+def test_locks_counted_only_where_taken(ctx, lock, mode):
+    n = 5000
+    # pairs: the forest is complete after the first iteration, in which no component is shared;
+    # a path of alternating weights is pairs after it, and takes more iterations
+    pairs = sym(n, np.arange(0, n, 2), np.arange(1, n, 2), np.arange(n // 2) % 9)
+    path = sym(n, np.arange(n - 1), np.arange(1, n), np.arange(n - 1) % 2)
+    for g, locked in ((pairs, False), (path, True)):
+        dg = ctx.load(g)
+        _, st = ctx.msf(dg, mode=mode, lock=lock)
+        assert (st["locks"] > 0) == locked
+        assert st["edges"] == (n - 1 if locked else n // 2)
+        dg.close()
