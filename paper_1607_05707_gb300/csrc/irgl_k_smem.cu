@@ -14,13 +14,16 @@
 // the pops differs, which the unique fixed point does not see.
 //
 // What bounds it: the round's chain of dependent shared-memory reads and atomics
-// (about 30 and 100 cycles each) and its barrier. So a round has one barrier (three
-// list counters in turn), a warp's pushes one atomic, and a frontier of up to 256
-// items gives every item four lanes, dealt across the warps; larger ones have their
-// edges dealt to the lanes by a scan. 64 x 64 grid BFS, 113 rounds: 1.1 us a round
-// and 128 us a call before, 0.65 and 99.5 us with these (narrow rounds below); R-MAT of
-// 2^10 vertices, SSSP: 97 -> 62 us (rounds of 360-525 items 5-10 us before, and 13 us went to 1024 threads
-// adding their edge counts to one 64-bit word).
+// (about 30 and 100 cycles each) and its barrier; with over a thousand items also the
+// one SM's instruction issue. So a round has one barrier (three list counters in turn),
+// and a frontier of up to 256 items gives every item four lanes, dealt across the warps.
+// Above that a lane walks a list of its own, in worklist order where no list of the graph
+// is long (neighbours in memory stay neighbours in the banks), and lists of more than
+// eight edges are dealt to the warp's lanes by a scan. Before -> now, each a call and the
+// wait for it: 64 x 64 grid BFS 179 -> 107 us (narrow rounds below included), its min-label
+// CC 373 -> 332; R-MAT of 2^10 vertices SSSP 95 -> 56; CC of a path of 3000 vertices 4.2 ->
+// 4.0 ms. With every list dealt by the scan, CC took 633 us and 11.2 ms; with the items
+// of R-MAT rounds in worklist order SSSP took 65 us.
 //
 // Shared-memory layout (32-bit words): row_ptr[n + 1], col[m], w[m] (SSSP),
 // value[n], stamp[n] (SSSP and CC: the round that last pushed the vertex, so
@@ -35,12 +38,13 @@ namespace {
 
 constexpr int kSmemCta = 1024;
 constexpr uint32_t kSmemWarps = kSmemCta / 32;
+constexpr uint32_t kSmemLane = 8;               // a lane walks lists of at most this many edges itself
 constexpr uint32_t kSmemFour = kSmemCta / 4;  // frontiers of at most this many items give each four lanes
 // Narrow rounds: a frontier of at most 64 items is one pass of eight warps, which cross a
 // barrier of their own faster than 32 warps cross the CTA's; the others wait at the next
-// CTA barrier until a frontier outgrows them (64 x 64 grid BFS 104 -> 87
-// us a call, SSSP on a 20 x 24 mesh 51 -> 42; 256 threads for the whole run instead
-// slow down wider frontiers: SSSP on a 50 x 60 mesh 89 -> 110).
+// CTA barrier until a frontier outgrows them (64 x 64 grid BFS 104 -> 87 us a call without
+// the wait, SSSP on a 20 x 24 mesh 51 -> 42; 256 threads for the whole run instead slow
+// down wider frontiers: SSSP on a 50 x 60 mesh 89 -> 110).
 constexpr uint32_t kNarrowWarps = 8;
 constexpr uint32_t kNarrow = kNarrowWarps * 8;
 
@@ -76,6 +80,20 @@ __device__ __forceinline__ bool smem_relax(const uint32_t* w, uint32_t* val_arr,
   if (OP == OP_BFS) return val_arr[v] == kInf && atomicCAS(val_arr + v, kInf, val) == kInf;
   const uint32_t nd = OP == OP_SSSP ? val + w[k] : val;
   return nd < val_arr[v] && nd < atomicMin(val_arr + v, nd) && atomicExch(stamp + v, r) != r;
+}
+
+// A short list [b, e) walked by one lane.
+template <uint32_t OP>
+__device__ __forceinline__ void smem_walk(const uint32_t* col, const uint32_t* w, uint32_t* val_arr, uint32_t* stamp,
+                                          uint32_t b, uint32_t e, uint32_t val, uint32_t r, uint32_t* out, uint32_t* out_n,
+                                          uint32_t cap, uint32_t* err) {
+  for (uint32_t k = b; k < e; ++k) {
+    const uint32_t v = col[k];
+    if (!smem_relax<OP>(w, val_arr, stamp, k, v, val, r)) continue;
+    const uint32_t pos = atomicAdd(out_n, 1u);  // one instruction for the lanes that are here together
+    if (pos < cap) out[pos] = v;
+    else atomicCAS(err, DERR_NONE, DERR_WL_OVERFLOW);
+  }
 }
 
 // A round over at most 8 * warps items by `warps` warps: four lanes per item, items
@@ -169,7 +187,9 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
     }
     smem_push(wl0, &s_n[0], n, push, s, &s_err);
   }
-  __syncthreads();
+  bool any_long = false;
+  for (uint32_t v = tid; v < n; v += kSmemCta) any_long |= rp[v + 1] - rp[v] > kSmemLane;
+  const bool longs = __syncthreads_or(any_long) != 0;
   trace_prologue(p.trace, p.trace_cap, t_start, s_n[0]);
   const uint32_t warp = tid >> 5;
   uint32_t edges = 0, rounds = 0, last_out = 0;
@@ -215,11 +235,20 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
     if (tid == 0) s_n[(r + 2) % 3] = 0;
     if (in_n <= kSmemFour) {
       edges += smem_four<OP>(in, in_n, kSmemWarps, rp, col, w, val, stamp, r, out, out_n, n, &s_err);
+    } else if (!longs) {
+      // every list is short: items in worklist order, one per lane, which walks its list
+      for (uint32_t i = tid; i < in_n; i += kSmemCta) {
+        const uint32_t u = in[i], b = rp[u], e = rp[u + 1];
+        smem_walk<OP>(col, w, val, stamp, b, e, OP == OP_BFS ? r + 1u : val[u], r, out, out_n, n, &s_err);
+        edges += e - b;
+      }
     } else {
-      // The warp's items (dealt across the warps) have their edges dealt out to
-      // its lanes, two per lane and step, owners by a shuffle search
+      // lists of at most kSmemLane edges by the lane that holds the item; the longer
+      // ones of the warp (items dealt across the warps, or in worklist order when there
+      // is more than one per thread) have their edges dealt out to its lanes, two per
+      // lane and step, owners by a shuffle search
       for (uint32_t base = 0; base < in_n; base += kSmemCta) {
-        const uint32_t i = base + lane * kSmemWarps + warp;
+        const uint32_t i = base + (in_n > kSmemCta ? tid : lane * kSmemWarps + ((warp + lane) & (kSmemWarps - 1u)));
         uint32_t b = 0, d = 0, x = 0;
         if (i < in_n) {
           const uint32_t u = in[i];
@@ -228,6 +257,13 @@ __global__ void __launch_bounds__(kSmemCta, 1) k_smem_iterate(KParams p) {
           x = OP == OP_BFS ? r + 1u : val[u];
         }
         edges += d;
+        const unsigned lng = __ballot_sync(kFull, d > kSmemLane);
+        if (d <= kSmemLane) {
+          smem_walk<OP>(col, w, val, stamp, b, b + d, x, r, out, out_n, n, &s_err);
+          d = 0;
+        }
+        __syncwarp();
+        if (lng == 0) continue;
         const uint32_t incl = warp_incl_scan(d), excl = incl - d;
         const uint32_t total = __shfl_sync(kFull, incl, 31);
         for (uint32_t s = 0; s < total; s += 64) {
