@@ -1557,6 +1557,13 @@ __device__ __forceinline__ void push_local(const V& g, Smem<CTA>& sm, const Roun
 // mesh a frontier grows by a few vertices per hop, on a power-law graph by orders.
 // 1021 x 1031 mesh, delta 1024, a source near a corner: 1883 rounds of 7.7 us and 16.4 ms
 // before, 4.6 ms now; 300 x 310: 4.6 and 1.15 ms; R-MAT of 2^18 vertices unchanged.
+// Sub-rounds that the caller asked for stop the same way, with CTA / 2 in kNearGrow's
+// place: their frontiers reach CTA items per CTA, and the CTAs of a mesh with 1024 threads
+// hold hundreds. Without it one CTA walked thousands of items alone, 32 at a time, and
+// passed on far more than its share (15 sub-rounds asked for: random graph of 2^14 vertices,
+// 4 entries each, BFS 428 us, 83 with it; R-MAT of 2^18, 4 each, SSSP 742 and 440; 24 R-MAT graphs
+// in a batch, BFS 1.9 and 0.65 ms); CTA in its place 74, 452 us and 0.77 ms, 2 * CTA 73, 604
+// and 0.94; meshes are the same with all three. Before local_round: 104 us, 543 us, 0.91 ms.
 constexpr uint32_t kNearLocal = 64, kNearGrow = 64, kLocalFar = 512;
 
 template <uint32_t OP, int CTA, class V>
@@ -1640,6 +1647,7 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
     if (want && pos < kLocalFar) s_far[kNearFarOp<OP> ? pos : 0u] = v;
     if (base + cnt > kLocalFar) push_far4<CTA>(sm, rc.far_out, want && pos >= kLocalFar ? 1u : 0u, v, 0u, 0u, 0u, nd);
   };
+  constexpr uint32_t grow = kNearFarOp<OP> ? kNearGrow : CTA / 2;
   uint32_t j = 0;
   for (; j <= rc.local_rounds; ++j) {
     const uint32_t n = min(l_n[j % 3], C);
@@ -1762,7 +1770,7 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
       }
     }
     __syncthreads();
-    if (kNearFarOp<OP> && l_n[(j + 1) % 3] > kNearGrow + 2u * m) {  // CTA-uniform: read after the barrier
+    if (l_n[(j + 1) % 3] > grow + 2u * m) {  // CTA-uniform: read after the barrier
       ++j;
       break;
     }
