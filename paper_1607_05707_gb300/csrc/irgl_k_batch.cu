@@ -4,7 +4,9 @@
 
 namespace irgl {
 
-// NF: near-far may be on; LOCAL: CTA-local sub-rounds (with or without near-far).
+// NF: near-far may be on; LOCAL: CTA-local sub-rounds. Sub-rounds without near-far have a
+// kernel of their own: in the one with both, min-label CC of 24 meshes of 0.2 M vertices took
+// 25.8 ms, 23.8 in its own (SSSP 12.7 and 12.2 ms).
 template <int CTA, bool NF, bool LOCAL>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_batch_iterate(BParams p) {
   __shared__ BatchSmem<CTA, NF> bs;
@@ -37,7 +39,9 @@ cudaError_t launch_b(uint32_t grid, const BParams& p, cudaStream_t s) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (p.local_rounds != 0) return cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, true, true>, p);
+  if (p.local_rounds != 0)
+    return p.delta != 0 ? cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, true, true>, p)
+                        : cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, false, true>, p);
   return p.delta != 0 ? cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, true, false>, p)
                       : cudaLaunchKernelEx(&cfg, k_batch_iterate<CTA, false, false>, p);
 }
@@ -66,7 +70,8 @@ cudaError_t occ_b(uint32_t cta, int* nb) {
 }
 
 cudaError_t occupancy_batch(uint32_t cta, bool near_far, bool local, int* nb) {
-  return local ? occ_b<true, true>(cta, nb) : near_far ? occ_b<true, false>(cta, nb) : occ_b<false, false>(cta, nb);
+  if (local) return near_far ? occ_b<true, true>(cta, nb) : occ_b<false, true>(cta, nb);
+  return near_far ? occ_b<true, false>(cta, nb) : occ_b<false, false>(cta, nb);
 }
 
 cudaError_t launch_extract_values(const unsigned long long* ds, uint32_t* out, uint64_t n, uint32_t grid,
