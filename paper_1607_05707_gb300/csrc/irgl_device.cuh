@@ -790,54 +790,57 @@ __device__ __forceinline__ uint32_t load_cur(const RoundCtx& rc, const uint32_t*
 }
 
 // Union-find over parent[] (parent[x] <= x, roots point at themselves), in
-// global or (SH) shared memory. Parents only ever move to smaller ancestors, so
-// every loop below ends. Global reads go through L1: a stale parent is still an
-// ancestor, and the CAS that hooks a root decides on the current value; read from
-// L2, the few roots of a large component are one line that every warp of the grid
-// queues for. uf_climb: the root above x, whose parent was read as `f`, halving
-// the path on the way (only non-roots are written, and only with their ancestors,
-// so a lost store just leaves a longer path).
+// global or (SH) shared memory. Parents only ever move to ancestors, which are
+// smaller, so every loop below ends. Global reads go through L1: a stale parent is
+// still an ancestor, and the CAS that hooks a root decides on the current value.
 template <bool SH>
 __device__ __forceinline__ uint32_t uf_ld(const uint32_t* p) {
   return SH ? *reinterpret_cast<const volatile uint32_t*>(p) : __ldca(p);
 }
-template <bool SH>
-__device__ __forceinline__ uint32_t uf_climb(uint32_t* parent, uint32_t x, uint32_t f) {
-  uint32_t prev = x;
-  while (f != prev) {
-    const uint32_t up = uf_ld<SH>(parent + f);
+
+// The root above x in a shared-memory tile, halving the path on the way (only non-roots
+// are written, and only with their ancestors: a lost store just leaves a longer path).
+__device__ __forceinline__ uint32_t uf_climb(uint32_t* tile, uint32_t x) {
+  volatile uint32_t* const t = tile;
+  uint32_t f = t[x];
+  while (f != x) {
+    const uint32_t up = t[f];
     if (up == f) return f;
-    if (SH) *reinterpret_cast<volatile uint32_t*>(parent + prev) = up;
-    else __stcg(parent + prev, up);
-    prev = f;
+    t[x] = up;
+    x = f;
     f = up;
   }
   return f;
 }
 
-// Join the trees of a and of rb, a (possibly former) root: the larger root is
-// hooked under the smaller one by a CAS that succeeds only on a root; a failed CAS
-// tells the parent it got meanwhile, and the climb from there reads L2.
-// Returns the joined tree's smaller end, an ancestor of a.
+// Join the trees of a and b, any two vertices: the larger one, if it is a root, is put
+// under the smaller one by a CAS, else its parent takes its place. The smaller one need
+// not be a root: it is not below the larger one, the smallest vertex of its own tree, so
+// nothing reads the few roots that everything ends up under (climbing to both roots
+// first, a random graph of 2^20 vertices with two entries each took 370-900 us, 190
+// like this; its random-id mesh 534 and 265). Returns a vertex of the joined tree, no
+// larger than a or b.
 template <bool SH>
-__device__ __forceinline__ uint32_t uf_link(uint32_t* parent, uint32_t a, uint32_t rb, uint32_t& hooked) {
-  uint32_t ra = uf_climb<SH>(parent, a, uf_ld<SH>(parent + a));
-  while (ra != rb) {
-    const uint32_t hi = max(ra, rb), lo = min(ra, rb);
-    uint32_t old = atomicCAS(parent + hi, hi, lo);
-    if (old == hi) {
-      ++hooked;
-      return lo;
+__device__ __forceinline__ uint32_t uf_link(uint32_t* parent, uint32_t a, uint32_t b, uint32_t& hooked) {
+  while (a != b) {
+    const uint32_t hi = max(a, b), lo = min(a, b);
+    uint32_t f = uf_ld<SH>(parent + hi);
+    if (f == hi) {
+      f = atomicCAS(parent + hi, hi, lo);
+      if (f == hi) {
+        ++hooked;
+        return lo;
+      }
     }
-    for (;;) {
-      const uint32_t up = SH ? uf_ld<SH>(parent + old) : __ldcg(parent + old);
-      if (up == old) break;
-      old = up;
+    const uint32_t up = uf_ld<SH>(parent + f);
+    if (up != f) {
+      if (SH) *reinterpret_cast<volatile uint32_t*>(parent + hi) = up;
+      else __stcg(parent + hi, up);
     }
-    ra = old;
-    rb = lo;
+    a = up;
+    b = lo;
   }
-  return ra;
+  return a;
 }
 
 // decide() with the near-far routing (SSSP, CC): 0 = no push, 1 = push to this
@@ -851,7 +854,7 @@ __device__ __forceinline__ uint32_t decide_route(uint32_t op_rt, uint32_t* state
   if (OP == OP_CCJ) {
     // link the roots of u (= val) and v; each edge is taken from its larger end
     uint32_t hooked = 0;
-    if (v < val) uf_link<false>(state, val, uf_climb<false>(state, v, cur), hooked);
+    if (v < val) uf_link<false>(state, val, cur, hooked);
     if (hooked) atomicAdd(rc.changes, 1u);
     return 0u;
   }
@@ -2979,72 +2982,101 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
 
 // Connected components by hooking and pointer jumping, in one cooperative
 // launch. parent = state; parent[v] <= v always, a root is parent[v] == v, and
-// every link puts the larger of two roots under the smaller one (uf_link), so the
+// every link puts a root under a smaller vertex of another tree (uf_link), so the
 // root of a tree is its smallest id. Every edge is taken from its larger end (a
 // symmetric graph holds both directions). Round 1: (a) each CTA takes blocks of
 // consecutive vertices, links the edges that stay inside a block in shared memory
 // and writes every vertex's parent, its block root; (b) after a barrier the edges
-// that leave a block downwards are linked in global memory. Round 2: every vertex
-// follows its parents to the root and stores it (skipped when nothing was hooked).
+// that leave a block downwards are linked in global memory, by whichever CTA. Round 2:
+// every vertex follows its parents to the root and stores it (skipped when nothing was
+// hooked).
 //
 // What bounds it: the adjacency is streamed twice; the rest is chains of dependent
-// parent reads, and they are what costs: with every link in global memory a
-// 4096^2 mesh (a tenth of its edges missing) took 2.9 ms, 25 us per warp step, the
-// rows of a wave climbing through each other; one parent per hook and iteration
-// (the former kernel: four iterations of 0.42-1.23 ms) 2.83 ms; with blocks of
-// nine rows in shared memory (a climb step is 30 cycles, and one edge in eighteen
-// leaves its block) 0.44 ms: 0.23 for (a), 0.18 for (b), 0.03 for round 2.
+// parent reads, and they are what costs: with every link in global memory a 4096^2
+// mesh (a tenth of its edges missing) took 2.9 ms, one parent per hook and iteration
+// (the former kernel: four iterations of 0.42-1.23 ms) 2.83 ms; with blocks of nine
+// rows in shared memory (a step is 30 cycles there, and one edge in eighteen leaves
+// its block) 0.45 ms: 0.26 for (a), 0.15 for (b), 0.04 for round 2. The former kernel's
+// call on the left, this one's on the right, in us: the same mesh with random ids 7190
+// and 1680, 1024^2 mesh with random ids 548 and 173, random graphs of 2^20 vertices with
+// 2, 6 and 32 entries each 372 / 184, 816 / 232 and 825 / 508, symmetric R-MAT of 2^16, 2^20 and
+// 2^22 vertices 190 / 106, 555 / 357 and 1700 / 960, 2^13 vertices of 127 entries 111 / 93, a path
+// of 2^20 in id order 1000 / 62.
 // Lists of at most kUfLane edges are walked by the lane that holds the vertex,
 // four columns in flight (no search for an edge's owner: mesh lists have two to
-// four entries); longer ones by the warp; those of kUfSplit edges or more by the
-// whole grid (big list), block edges included.
+// four entries); the longer ones of a warp have their edges dealt to its lanes, four
+// each in flight (one list at a time instead, the random graph of 32 entries took 950 us);
+// those of kUfSplit edges or more are dealt to the whole grid (big list), block edges
+// included.
 constexpr uint32_t kUfLane = 16;
 constexpr uint32_t kUfSplit = 512;
+constexpr uint32_t kUfSliced = 1u << 17;  // vertices from which the second neighbours are linked in slices
 constexpr int kUfCta = 1024;
 constexpr uint32_t kUfTile = 40 * 1024;  // vertices of a block: 160 KB of shared memory beside the CTA's Smem
 
-// Vertices per block: the smallest number of blocks that is a multiple of the
-// grid and fits the tile (no CTA is left with one block more than the others),
-// but at least 1024, so that a small graph keeps some of its edges inside blocks.
-__device__ __forceinline__ uint32_t uf_block_size(uint32_t n, uint32_t grid) {
+// Vertices per block, a multiple of a warp's: the smallest number of blocks that is a
+// multiple of the grid and fits the tile (no CTA is left with one block more than the
+// others), but at least 1024, or what holds 16 K adjacency entries, so that a small graph
+// keeps some of its edges inside blocks (2^13 vertices of 127 entries: eight blocks of 1024
+// left 144 CTAs idle, 190 us a call).
+__device__ __forceinline__ uint32_t uf_block_size(uint32_t n, uint32_t m, uint32_t grid) {
   const unsigned long long tiles = static_cast<unsigned long long>(kUfTile) * grid;
   const unsigned long long nb = max((n + tiles - 1u) / tiles, 1ull) * grid;
-  return min(max(static_cast<uint32_t>((n + nb - 1u) / nb), 1024u), kUfTile);
+  const unsigned long long most = (16384ull * n) / max(m, 1u);  // vertices of 16 K entries
+  const uint32_t least = static_cast<uint32_t>(min(max(most, 32ull), 1024ull));
+  return (min(max(static_cast<uint32_t>((n + nb - 1u) / nb), least), kUfTile) + 31u) & ~31u;
 }
 
-// Link the edges (u, v) of the vertices [lo, hi): inside the block (SH: v >= lo,
-// parents tile[] indexed from lo) or below it (v < lo, parents in p.state).
+// Vertices that one of `warps` warps takes at a time of n: 32, or fewer (a power of
+// two) where n leaves warps without any.
+__device__ __forceinline__ uint32_t uf_share(uint32_t n, unsigned long long warps) {
+  uint32_t vp = 32;
+  while (vp > 1u && n <= warps * (vp >> 1)) vp >>= 1;
+  return vp;
+}
+
+// Link edges (u, v) of the vertices below hi that this warp takes (the `share` of them
+// at `first`, then every `stride`): inside the block that starts at lo (SH: v >= lo,
+// parents tile[] indexed from lo) or leaving their block of bs vertices downwards
+// (v below it, parents in p.state).
 template <bool SH>
-__device__ __forceinline__ void uf_edges(const KParams& p, Smem<kUfCta>& sm, const RoundCtx& rc, uint32_t lo, uint32_t hi,
+__device__ __forceinline__ void uf_edges(const KParams& p, Smem<kUfCta>& sm, const RoundCtx& rc, uint32_t lo, uint32_t bs,
+                                         uint32_t hi, unsigned long long first, unsigned long long stride, uint32_t share,
                                          uint32_t split, uint32_t* tile, uint32_t& edges, uint32_t& hooked) {
+  // edges: entries of the lists walked (SH: of those, the ones that stay inside the block)
   const uint32_t lane = threadIdx.x & 31;
   uint32_t* const par = SH ? tile : p.state;
   const uint32_t off = SH ? lo : 0u;
-  uint32_t nbeg = threadIdx.x < hi - lo ? __ldg(p.row_ptr + lo + threadIdx.x) : 0u;
-  uint32_t nend = threadIdx.x < hi - lo ? __ldg(p.row_ptr + lo + threadIdx.x + 1) : 0u;
-  for (uint32_t base = threadIdx.x & ~31u; base < hi - lo; base += kUfCta) {
-    const uint32_t u = lo + base + lane;
+  uint32_t nbeg = 0, nend = 0;
+  if (lane < share && first + lane < hi) {
+    nbeg = __ldg(p.row_ptr + first + lane);
+    nend = __ldg(p.row_ptr + first + lane + 1);
+  }
+  for (unsigned long long base = first; base < hi; base += stride) {
+    const uint32_t u = static_cast<uint32_t>(base) + lane;  // lanes past the share or the end hold an empty list
     const uint32_t beg = nbeg, end = nend;
-    const bool more = base + kUfCta + lane < hi - lo;  // the next step's offsets, loaded a step ahead
-    nbeg = more ? __ldg(p.row_ptr + u + kUfCta) : 0u;
-    nend = more ? __ldg(p.row_ptr + u + kUfCta + 1) : 0u;
+    const bool more = lane < share && base + stride + lane < hi;  // the next step's offsets, loaded a step ahead
+    nbeg = more ? __ldg(p.row_ptr + base + stride + lane) : 0u;
+    nend = more ? __ldg(p.row_ptr + base + stride + lane + 1) : 0u;
+    if (!SH) lo = static_cast<uint32_t>(base) / bs * bs;
     const uint32_t deg = end - beg;
     if (!SH) edges += deg;
     bool wide = deg > kUfLane;
+    uint32_t ru = SH ? u - off : deg != 0 ? uf_ld<false>(par + u) : 0u;
     if (!wide) {
-      uint32_t ru = u - off;
-      for (uint32_t e = beg; e < end; e += 4) {
+      for (uint32_t e = 0; e < deg; e += 4) {
         uint32_t c[4], f[4];
 #pragma unroll
         for (uint32_t k = 0; k < 4; ++k) {
-          c[k] = e + k < end ? __ldg(p.col + e + k) : kInf;
+          c[k] = e + k < deg ? __ldg(p.col + beg + e + k) : kInf;
           if (SH ? (c[k] < lo || c[k] >= u) : c[k] >= lo) c[k] = kInf;
         }
 #pragma unroll
         for (uint32_t k = 0; k < 4; ++k) f[k] = c[k] != kInf ? uf_ld<SH>(par + (c[k] - off)) : 0u;
+        if (SH) edges += (c[0] != kInf) + (c[1] != kInf) + (c[2] != kInf) + (c[3] != kInf);
 #pragma unroll
         for (uint32_t k = 0; k < 4; ++k)
-          if (c[k] != kInf) ru = uf_link<SH>(par, ru, uf_climb<SH>(par, c[k] - off, f[k]), hooked);
+          if (c[k] != kInf && f[k] != ru) ru = uf_link<SH>(par, ru, f[k], hooked);
       }
     }
     // lists for the whole grid: listed once (in the global pass), with every edge they have
@@ -3070,18 +3102,32 @@ __device__ __forceinline__ void uf_edges(const KParams& p, Smem<kUfCta>& sm, con
         }
       }
     }
-    for (unsigned m = __ballot_sync(kFull, wide); m; m &= m - 1) {
-      const int ld = __ffs(m) - 1;
-      const uint32_t wu = __shfl_sync(kFull, u, ld);
-      const uint32_t we = __shfl_sync(kFull, end, ld);
-      // a listed vertex that found the big list full walks its block edges here too
-      const uint32_t top = SH ? wu : (__shfl_sync(kFull, big ? 1u : 0u, ld) ? wu : lo);
-      uint32_t ru = wu - off;
-      for (uint32_t e = __shfl_sync(kFull, beg, ld) + lane; e < we; e += 32) {
-        const uint32_t v = ld_adj(p.col + e);
-        if (v < top && (!SH || v >= lo))
-          ru = uf_link<SH>(par, ru, uf_climb<SH>(par, v - off, uf_ld<SH>(par + (v - off))), hooked);
+    if (!__any_sync(kFull, wide)) continue;
+    // the wide lists' edges (fewer than 2^32 in all) dealt to the lanes, four in flight each
+    const uint32_t top = SH || big ? u : lo;  // a vertex that found the big list full walks its block edges here too
+    const uint32_t d = wide ? deg : 0u;
+    const uint32_t incl = warp_incl_scan(d), excl = incl - d;
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+    for (unsigned long long s = 0; s < total; s += 128) {
+      uint32_t c[4], f[4], a[4];
+      if (wide) ru = uf_ld<SH>(par + ru);
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) {
+        const bool in = s + 32u * k + lane < total;
+        const uint32_t e = in ? static_cast<uint32_t>(s) + 32u * k + lane : total - 1u;
+        const uint32_t own = warp_find<uint32_t>(excl, e, 32);
+        const uint32_t at = __shfl_sync(kFull, beg - excl, own) + e;
+        const uint32_t below = __shfl_sync(kFull, top, own);
+        a[k] = __shfl_sync(kFull, ru, own);
+        c[k] = in ? ld_adj(p.col + at) : kInf;
+        if (c[k] >= below || (SH && c[k] < lo)) c[k] = kInf;
       }
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) f[k] = c[k] != kInf ? uf_ld<SH>(par + (c[k] - off)) : 0u;
+      if (SH) edges += (c[0] != kInf) + (c[1] != kInf) + (c[2] != kInf) + (c[3] != kInf);
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k)
+        if (c[k] != kInf && f[k] != a[k]) uf_link<SH>(par, a[k], f[k], hooked);
     }
   }
 }
@@ -3116,35 +3162,33 @@ __device__ __forceinline__ void cc_jump_persistent(const KParams& p, Smem<kUfCta
   if (p.skip_cta == static_cast<int>(blockIdx.x)) return;  // test hook: never arrives
   SingleView<OP_CCJ> g{p.row_ptr, p.col, p.w, p.state, p.stamp, p.n};
   const unsigned long long t_run0 = p.time_limit_ns ? globaltimer_ns() : 0ull;
-  uint32_t edges = 0, rounds = 0, hooks = 0, hooked = 0;
+  uint32_t edges = 0, inside = 0, rounds = 0, hooks = 0, hooked = 0;
   const uint32_t split = max(p.tn.cta_thresh, kUfSplit);
-  const uint32_t bs = uf_block_size(p.n, gridDim.x);
+  const uint32_t m = __ldg(p.row_ptr + p.n), bs = uf_block_size(p.n, m, gridDim.x);
   const uint32_t nblocks = p.n / bs + (p.n % bs != 0 ? 1u : 0u);
-  RoundCtx rc;
+  const uint32_t warp = threadIdx.x >> 5;
+  RoundCtx rc{};
   rc.out = Out{p.items[0], &st->tail[1], p.cap, &st->err};  // never pushed
   rc.big = p.big;
   rc.big_ctr = &st->big_ctr;
   rc.limit = kInf;
-  rc.ds = nullptr;
-  rc.vis = nullptr;
-  rc.mf = nullptr;
   rc.changes = &sm.round_pushes;  // the barrier publishes the grid's sum
   for (uint32_t b = blockIdx.x; b < nblocks; b += gridDim.x) {
     const uint32_t lo = b * bs, hi = lo + min(bs, p.n - lo);
     for (uint32_t i = threadIdx.x; i < hi - lo; i += CTA) tile[i] = i;
     __syncthreads();
-    uf_edges<true>(p, sm, rc, lo, hi, split, tile, edges, hooked);
+    const uint32_t share = uf_share(hi - lo, CTA / 32);
+    uf_edges<true>(p, sm, rc, lo, bs, hi, static_cast<unsigned long long>(lo) + warp * share, CTA / 32 * share, share, split, tile,
+                   inside, hooked);
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < hi - lo; i += CTA) {
-      uint32_t x = tile[i];
-      for (uint32_t y = tile[x]; y != x; y = tile[x]) x = y;
-      __stcg(p.state + lo + i, lo + x);
-    }
+    // halving the paths on the way: a block that is one path can be as deep as it has
+    // vertices (2^20-vertex path 828 us without, 62 with; a mesh pays 2 % for the writes)
+    for (uint32_t i = threadIdx.x; i < hi - lo; i += CTA) __stcg(p.state + lo + i, lo + uf_climb(tile, i));
     __syncthreads();
   }
-  if (hooked) atomicAdd(rc.changes, hooked);
+  if (inside) atomicAdd(rc.changes, inside);
   bool ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
-  hooks = sm.pub_out;
+  hooks = sm.pub_out;  // no edge inside a block, no root hooked yet
   trace_round(p.trace, p.trace_cap, 0, p.n, hooks);
   if (ok) {
     if (threadIdx.x == 0) {
@@ -3154,26 +3198,33 @@ __device__ __forceinline__ void cc_jump_persistent(const KParams& p, Smem<kUfCta
     __syncthreads();
     check_time_limit(&st->err, t_run0, p.time_limit_ns);
     hooked = 0;
-    if (hooks < p.n / 2) {
-      // few edges stayed inside a block (ids without locality): link two neighbours
-      // of every vertex first and flatten, so that most of the edges below find both
-      // ends under one root and cost one read, instead of all racing to hook the
-      // same few roots (symmetric R-MAT, 2^16 vertices, 1.8 M entries: 142 us a call, the
-      // former kernel 311; 2^20, 31 M: 846, without this 770-1056, former 907-2421)
-      for (unsigned long long i = blockIdx.x * CTA + threadIdx.x; i < p.n; i += gridDim.x * CTA) {
-        const uint32_t u = static_cast<uint32_t>(i);
-        const uint32_t beg = __ldg(p.row_ptr + u), end = min(__ldg(p.row_ptr + u + 1), beg + 2u);
-        uint32_t ru = u;
-        for (uint32_t e = beg; e < end; ++e) {
-          const uint32_t v = __ldg(p.col + e);
-          if (v < p.n) ru = uf_link<false>(p.state, ru, uf_climb<false>(p.state, v, __ldca(p.state + v)), hooked);
+    if (hooks < m / 8) {
+      // Few edges stay inside a block (ids without locality; half of the entries are
+      // looked at, from the larger end): link two neighbours of every vertex first
+      // (neighbour sampling as in Sutton, Ben-Nun and Barak's Afforest, IPDPS 2018),
+      // flattening after each, so that most of the edges below find both ends under one
+      // root and cost one read, instead of all racing to hook the same few roots. The
+      // second neighbours make one large tree of the small ones, in chains that get
+      // longer while nothing flattens them: a quarter, a quarter and half of them at a
+      // time take the random graph of 2^17 vertices with 4 entries each from 224 to 90 us
+      // and the 1024^2 random-id mesh from 277 to 173; below 2^17 vertices the four more
+      // barriers cost more than that (R-MAT of 2^16 104 us, 116 in slices).
+      const uint32_t passes = p.n >= kUfSliced ? 4u : 2u;
+      for (uint32_t pass = 0; ok && pass < passes; ++pass) {
+        const uint32_t k = pass != 0 ? 1u : 0u;
+        const uint32_t from = pass > 1u ? p.n >> (passes - pass) : 0u, to = pass != 0 ? p.n >> (passes - 1u - pass) : p.n;
+        for (unsigned long long i = static_cast<unsigned long long>(from) + blockIdx.x * CTA + threadIdx.x; i < to;
+             i += static_cast<unsigned long long>(gridDim.x) * CTA) {
+          const uint32_t u = static_cast<uint32_t>(i), beg = __ldg(p.row_ptr + u);
+          if (__ldg(p.row_ptr + u + 1) - beg <= k) continue;
+          const uint32_t v = __ldg(p.col + beg + k), f = __ldca(p.state + v), ru = __ldca(p.state + u);
+          if (f != ru) uf_link<false>(p.state, ru, f, hooked);
         }
-      }
-      if (hooked) atomicAdd(rc.changes, hooked);
-      hooked = 0;
-      ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
-      hooks |= sm.pub_out;
-      if (ok) {
+        if (hooked) atomicAdd(rc.changes, hooked);
+        hooked = 0;
+        ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
+        hooks |= sm.pub_out;
+        if (!ok) break;
         uf_flatten(p);
         if (threadIdx.x == 0) sm.round_pushes = 0;
         ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns);
@@ -3183,8 +3234,13 @@ __device__ __forceinline__ void cc_jump_persistent(const KParams& p, Smem<kUfCta
   if (ok) {
     if (threadIdx.x == 0) sm.round_pushes = 0;
     __syncthreads();
-    for (uint32_t b = blockIdx.x; b < nblocks; b += gridDim.x)
-      uf_edges<false>(p, sm, rc, b * bs, b * bs + min(bs, p.n - b * bs), split, tile, edges, hooked);
+    // every CTA takes a range of the vertices, whichever their blocks
+    const uint32_t share = uf_share(p.n, static_cast<unsigned long long>(gridDim.x) * (CTA / 32));
+    const uint32_t chunks = p.n / share + (p.n % share != 0 ? 1u : 0u);
+    const unsigned long long per = static_cast<unsigned long long>(chunks / gridDim.x + (chunks % gridDim.x != 0 ? 1u : 0u)) * share;
+    const unsigned long long from = blockIdx.x * per;
+    uf_edges<false>(p, sm, rc, 0u, bs, static_cast<uint32_t>(min(from + per, static_cast<unsigned long long>(p.n))), from + warp * share,
+                    CTA / 32 * share, share, split, tile, edges, hooked);
     if (hooked) atomicAdd(rc.changes, hooked);
     ok = grid_barrier<CTA>(sm, st, gen, p.timeout_ns, p.big.cap != 0);
     hooks |= sm.pub_out;
