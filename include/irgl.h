@@ -169,7 +169,8 @@ typedef struct {
   uint32_t grid;          /* CTAs per launch */
   uint32_t cta_size;      /* threads per CTA */
   uint32_t launches;      /* CUDA kernel launches issued by the call */
-  uint64_t edges_scanned; /* adjacency entries read, re-relaxations included */
+  uint64_t edges_scanned; /* adjacency entries read, re-relaxations included (IRGL_CC_JUMP: each
+                             entry once, whatever its passes read again) */
   uint32_t last_out;      /* size of the final out-worklist (0 when Iterate drained it) */
   float device_ms;        /* CUDA-event time of the call's launches, when the call measures it (else 0) */
 } irgl_stats;
