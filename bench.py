@@ -556,7 +556,7 @@ def run_gpu(args, world, rank, local):
                              us_per_round=1e6 * tk / max(1, sum(nrounds[k])),
                              work_inefficiency=scanned[k] / max(1, sum(counts[(j, k)][1] for j in set(used))))
     dom = max(kernels, key=lambda k: per_kernel[k]["time_s"])
-    kname = {"bfs": "k_iterate<BFS>", "sssp": "k_iterate<SSSP>", "cc": "k_iterate<CC>", "cc_jump": "k_iterate<CCJ>"}[dom]
+    kname = {"bfs": "k_iterate<BFS>", "sssp": "k_iterate<SSSP>", "cc": "k_iterate<CC>", "cc_jump": "k_cc_jump"}[dom]
     pk = per_kernel[dom]
     traffic = measured_traffic(kname, args.workload if args.workload != "rmat20" or args.scale == 20 else "")
     roofline = {"bound": "hbm", "achieved": round(pk["achieved_gbs"], 2), "peak": hbm, "unit": "GB/s",

@@ -1509,12 +1509,13 @@ __device__ __forceinline__ void process_tile(const V& g, Smem<CTA>& sm, const Ro
 // What bounds it: a chain of dependent reads per sub-round, not bandwidth (4096^2
 // mesh BFS: a few thousand items over 1216 CTAs). Through process_tile the chain
 // was row offsets -> column -> neighbour's word -> atomic, with a shuffle scan and
-// a search per edge between them: 3.3 us a sub-round. Here an entry carries its
-// row offsets (read beside the atomicMin that discovers it), a list is dealt to
-// four lanes without a search, and the atomicMin is issued without reading the
-// word first: two dependent reads are left, (own word | columns) -> (atomicMin |
-// the neighbour's row offsets). 4096^2 mesh BFS, 382 rounds of 16 sub-rounds: 54 -> 32 us
-// a round, 16.7 -> 9.9 ms a call; with a read before the atomicMin 11.2 ms.
+// a search per edge between them. Here an entry carries its row offsets (read beside
+// the atomicMin that discovers it), a list is dealt to four lanes without a search,
+// and the atomicMin is issued without reading the word first: two dependent reads are
+// left, (own word | columns) -> (atomicMin | the neighbour's row offsets). 4096^2 mesh
+// BFS, a call of 382 rounds of 16 sub-rounds, is 1.69 times as fast as through
+// process_tile (1.49 with a read before the atomicMin), 1.78 with the prefetches below:
+// 9.6 ms, 1.6 us a sub-round.
 //
 // Entries {item, first edge, end (, query)} live in two halves of the stage that
 // alternate; pushes that find a half full go straight to the out-worklist. Lists
@@ -1734,8 +1735,8 @@ __device__ __forceinline__ void local_round(const V& g, Smem<CTA>& sm, const Rou
         }
         if (push) {
           // what the next sub-rounds read if ids have locality: v's columns, and the words
-          // a line further on either side (4096^2 mesh BFS 12.25 -> 11.5 ms, columns alone
-          // 11.77, words alone 11.90)
+          // a line further on either side (4096^2 mesh BFS 6 % less time a call, columns alone
+          // 4 %, words alone 3 %)
           if (nb < ne) prefetch_l2(col + nb);
           if (v >= 16u) prefetch_l2(rc.ds + sb + v - 16u);
           if (v + 16u < nv) prefetch_l2(rc.ds + sb + v + 16u);
@@ -2780,12 +2781,12 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
       r0 = 1;
     }
   }
-  // small frontiers skip the big list (broadcast_round): BFS, SSSP and
-  // min-label CC rounds (near-far included) without CTA-local sub-rounds
   // near-far sub-rounds end for good with the first list long enough for the big list:
   // a graph that has those is not the mesh they are for (borrowed graphs' degrees are
   // not known to the host)
   bool near_local = LOCAL && kNearFarOp<OP>;
+  // small frontiers skip the big list (broadcast_round): BFS, SSSP and min-label CC
+  // (near-far included), in the rounds that take no sub-rounds
   const bool bcast_ok = p.bcast != 0 && (OP == OP_BFS || base_op(OP) == OP_SSSP || base_op(OP) == OP_CC);
   // dense rounds: BFS, and SSSP on packed words, without near-far or sub-rounds
   const bool dense_ok = p.dense_div != 0 && !nf && p.local_rounds == 0 &&
