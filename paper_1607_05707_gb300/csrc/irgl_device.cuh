@@ -429,14 +429,16 @@ struct Smem {
   uint8_t pushed[CTA];                      // ReduceAndReturn All: item pushed something
 };
 
-// Far items of a batched launch staged per CTA: the far list is appended with one
-// atomic per flush instead of one per pushing warp on its single counter. With the
+// Far items of a batched launch with sub-rounds are staged per CTA: the far list is
+// appended with one atomic per flush instead of one per pushing warp on its single
+// counter (in plain near-far rounds, which push few far items each, the flush at the
+// round's end is one more wait: 24 SSSP queries on meshes 27.4 ms, 26.5 without). With the
 // sparse round's even deal of the far items and limits that rise in the round that
 // drained a query, 91 SSSP queries on grids went from 332 rounds and 36 ms to 177
 // rounds and 12.5 ms.
 constexpr uint32_t kFarStage = 1024;
 
-template <int CTA, bool NF>
+template <int CTA, bool NF, bool STAGE>
 struct BatchSmem {
   Smem<CTA> core;
   uint32_t sbases[kMaxBatchQueries];
@@ -444,7 +446,7 @@ struct BatchSmem {
   uint32_t qfar[kMaxBatchQueries / 32];   // queries (by slot) active otherwise: items kept on the far
                                           // list, pushes already expanded by the sub-rounds
   uint32_t lim[NF ? kMaxBatchQueries : 1];  // near-far: this round's limit of each query (by id)
-  uint32_t far_stage[NF ? kFarStage : 1u];  // far items on their way to the far list
+  uint32_t far_stage[STAGE ? kFarStage : 1u];  // far items on their way to the far list
   uint32_t far_n;
   uint32_t dmin[NF ? 1 : kMaxBatchQueries];  // by slot: the smallest SSSP distance this CTA pushed this round
 };
@@ -625,10 +627,11 @@ struct SingleView {
 };
 
 // Many queries over many graphs; op taken per query at run time. NF: near-far
-// (per-query limits) may be on.
-template <bool NF>
+// (per-query limits) may be on. STAGE: far items go through the CTA's stage.
+template <bool NF, bool STAGE>
 struct BatchView {
   static constexpr bool kNear = NF;
+  static constexpr bool kStageFar = STAGE;
   const QDesc* __restrict__ desc;
   const uint32_t* sbases;  // shared-memory copy
   uint32_t nq;
@@ -1120,6 +1123,10 @@ __device__ __forceinline__ void push_far_item(const V& g, Smem<CTA>& sm, const R
     f = atomicExch(g.far_stamp + item, rc.ep) != rc.ep;
     g.mark_active(q);
   }
+  if constexpr (!V::kStageFar) {
+    push_far4<CTA>(sm, rc.far_out, f ? 1u : 0u, item, 0u, 0u, 0u, kInf);
+    return;
+  }
   const unsigned m = __ballot_sync(kFull, f);
   if (m == 0) return;
   const int ld = __ffs(m) - 1;
@@ -1137,6 +1144,7 @@ __device__ __forceinline__ void push_far_item(const V& g, Smem<CTA>& sm, const R
 // thread of the CTA, at a CTA-uniform point.
 template <int CTA, class V>
 __device__ __forceinline__ void flush_far(const V& g, Smem<CTA>& sm, const RoundCtx& rc, uint32_t above) {
+  if constexpr (!V::kStageFar) return;
   if (!__syncthreads_or(*g.far_n > above)) return;
   const uint32_t n = min(*g.far_n, kFarStage);
   if (threadIdx.x == 0) sm.gbase = atomicAdd(rc.far_out.tail, n);
@@ -3330,7 +3338,7 @@ __device__ __forceinline__ void invoke_round(const KParams& p, const RoundArgs& 
 // epoch); the launch stops when the worklist drains or after max_rounds
 // rounds (an epoch), leaving the pending items and their buffer in p.cont.
 template <int CTA, bool NF, bool LOCAL>
-__device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA, NF>& bs) {
+__device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA, NF, NF && LOCAL>& bs) {
   Smem<CTA>& sm = bs.core;
   init_smem<CTA>(sm);
   const uint32_t nq = min(p.nq, static_cast<uint32_t>(kMaxBatchQueries));
@@ -3350,7 +3358,7 @@ __device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA, N
   uint32_t far_n = nf ? min(__ldcg(p.cont + 3), p.far_cap) : 0u;
   if (nf)
     for (uint32_t i = threadIdx.x; i < nq; i += CTA) bs.lim[i] = __ldcg(p.blim + __ldg(&p.desc[i].slot));
-  BatchView<NF> g{p.desc, bs.sbases, nq, p.state, p.stamp, bs.qbits, bs.qfar, nf ? bs.lim : nullptr, p.far_stamp, bs.far_stage, &bs.far_n, bs.dmin};
+  BatchView<NF, NF && LOCAL> g{p.desc, bs.sbases, nq, p.state, p.stamp, bs.qbits, bs.qfar, nf ? bs.lim : nullptr, p.far_stamp, bs.far_stage, &bs.far_n, bs.dmin};
   if (threadIdx.x == 0) bs.far_n = 0;
   if (!NF && bdefer)
     for (uint32_t i = threadIdx.x; i < static_cast<uint32_t>(kMaxBatchQueries); i += CTA) bs.dmin[i] = kInf;

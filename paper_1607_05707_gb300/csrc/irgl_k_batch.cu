@@ -9,7 +9,7 @@ namespace irgl {
 // 25.8 ms, 23.8 in its own (SSSP 12.7 and 12.2 ms).
 template <int CTA, bool NF, bool LOCAL>
 __global__ void __launch_bounds__(CTA, MinBlocks<CTA>::value) k_batch_iterate(BParams p) {
-  __shared__ BatchSmem<CTA, NF> bs;
+  __shared__ BatchSmem<CTA, NF, NF && LOCAL> bs;
   iterate_batch<CTA, NF, LOCAL>(p, bs);
 }
 
