@@ -2070,8 +2070,11 @@ __device__ __forceinline__ unsigned long long arrive_add(unsigned long long* p, 
 // bounded by timeout_ns and gives up early when another CTA timed out. With
 // one CTA the barrier is just __syncthreads (a two-level arrival through
 // 32 group words measured 1.2 us slower per barrier on 1216 CTAs: the queue
-// of atomics on one word is not what a barrier waits for). The caller clears
-// sm.round_pushes and sm.big_appended at the start of each round.
+// of atomics on one word is not what a barrier waits for). The barrier that ends a
+// round clears the CTA's counters for the next one while the other threads wait: cleared
+// by thread 0 after the barrier, a warp that ran ahead of it could lose its big-list flag,
+// and with it the only long list of the round (SSSP with CTAs of 1024 on a graph with
+// three hubs: one run in a hundred kept a hub's former distance).
 template <int CTA>
 __device__ __forceinline__ bool grid_barrier(Smem<CTA>& sm, DevStatus* st, uint32_t& gen, unsigned long long timeout_ns,
                                              bool with_big = false) {
@@ -2138,6 +2141,12 @@ __device__ __forceinline__ bool grid_barrier(Smem<CTA>& sm, DevStatus* st, uint3
     sm.pub_err = flags & 0x7Fu;
     sm.pub_flags = flags & kRelBigFlag;
     sm.pub_big = big;
+    if ((flags & kRelBigFlag) == 0) {  // the round is over: the next one's counters start here
+      sm.round_pushes = 0;
+      sm.big_appended = 0;
+      sm.far_min_cta = kInf;
+      sm.mf_cta = 0;
+    }
   }
   __syncthreads();
   return sm.flag != 0;
@@ -2280,6 +2289,8 @@ __device__ __forceinline__ void init_smem(Smem<CTA>& sm) {
     sm.flag = 0;
     sm.round_pushes = 0;
     sm.big_appended = 0;
+    sm.far_min_cta = kInf;
+    sm.mf_cta = 0;
     sm.pmin_cta = kInf;
   }
   __syncthreads();
@@ -2858,10 +2869,6 @@ __device__ __forceinline__ void iterate_persistent(const KParams& p, Smem<CTA>& 
         st->tail[(r + 2) % 3] = 0;
         st->grab[(r + 2) % 3] = 0;
       }
-      sm.round_pushes = 0;
-      sm.big_appended = 0;
-      sm.far_min_cta = kInf;
-      sm.mf_cta = 0;
       // mf[(r + 2) % 3] is still being read by CTAs that just left the last
       // barrier; mf[(r + 1) % 3] was read by every CTA before it arrived there
       if (dopt && blockIdx.x == 0) st->mf[(r + 1) % 3] = 0;
@@ -3475,8 +3482,6 @@ __device__ __forceinline__ void iterate_batch(const BParams& p, BatchSmem<CTA, N
         st->tail[(r + 2) % 3] = 0;
         st->grab[(r + 2) % 3] = 0;
       }
-      sm.round_pushes = 0;
-      sm.big_appended = 0;
     }
     round_body<OP_RUNTIME, CTA, RED_NONE, LOCAL>(g, sm, rc, edges, dummy_t, dummy_f);
     fold_marks(r);
