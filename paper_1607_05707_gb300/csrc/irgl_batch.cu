@@ -333,10 +333,11 @@ irgl_status irgl_batch_prepare(irgl_batch* b, const irgl_tuning* tin, int use_cu
   }
   // worklists: one entry per arena vertex; with CTA-local sub-rounds a vertex
   // lowered again in a later sub-round of the same round can be on the next
-  // round's worklist twice, so they get twice the room (a round that still
-  // overflows reports IRGL_ERR_WL_OVERFLOW)
+  // round's worklist twice, so they get twice the room, and what every CTA can
+  // leave of its last sub-round (2048 entries an SM; a round that still overflows
+  // reports IRGL_ERR_WL_OVERFLOW)
   const bool sub = packed && ((t.flags >> 8) & 15u) != 0;
-  b->wl_cap = std::min<uint64_t>(b->arena_n * (sub ? 2u : 1u), 0xFFFFFFF0ull);
+  b->wl_cap = std::min<uint64_t>(b->arena_n * (sub ? 2u : 1u) + (sub ? 2048ull * static_cast<uint64_t>(ctx->sm_count) : 0ull), 0xFFFFFFF0ull);
   if (e == cudaSuccess) e = cudaMalloc(&b->items[0], sizeof(uint32_t) * b->wl_cap);
   if (e == cudaSuccess) e = cudaMalloc(&b->items[1], sizeof(uint32_t) * b->wl_cap);
   if (e == cudaSuccess) e = cudaMalloc(&b->qlast, sizeof(uint32_t) * Q);

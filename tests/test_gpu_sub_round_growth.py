@@ -55,3 +55,29 @@ def test_hub_at_the_bound(ctx, cta, over):
         np.testing.assert_array_equal(b.result(0)[0], want)
         b.close()
     dg.close()
+
+
+@pytest.mark.parametrize("flags", [0xF41, 0x101, 0x401])
+@pytest.mark.parametrize("cta", [128, 1024])
+def test_star_components_fit_the_worklists(ctx, flags, cta):
+    # a hub whose label falls again and again, each time pushing every leaf, in a batch of two
+    from paper_1607_05707_gb300.api import Batch
+
+    for seed in range(4):
+        rng = np.random.default_rng(seed)
+        n = int(rng.integers(3000, 9000))
+        p = rng.permutation(n)
+        u, v = np.full(n - 1, p[0]), p[1:]
+        g = inputs.csr_from_edges(n, np.concatenate([u, v]), np.concatenate([v, u]), symmetric=True)
+        dg = ctx.load(g)
+        want = oracle.cc(n, g.row_ptr, g.col)
+        b = Batch(ctx)
+        for _ in range(2):
+            b.add("cc", dg)
+        b.prepare(dict(cta_size=cta, flags=flags))
+        for _ in range(20):
+            b.run()
+            for r in b.results():
+                np.testing.assert_array_equal(r, want)
+        b.close()
+        dg.close()
