@@ -264,6 +264,7 @@ struct irgl_server {
   uint32_t grid = 0;
   uint32_t sub_rounds = 0;  // CTA-local sub-rounds of the batched kernel (packed arena only)
   uint32_t id_step = 1;     // round ids per round: 1 + sub_rounds
+  uint64_t wl_cap = 0;      // entries of each worklist
   irgl_tuning t{};
   Arena arena;
   std::vector<uint32_t> free_slots;
@@ -557,7 +558,7 @@ bool server_step(irgl_server* s) {
     ap.qfirst = s->qfirst;
     ap.items[0] = s->items[0];
     ap.items[1] = s->items[1];
-    ap.cap = static_cast<uint32_t>(s->arena_n);
+    ap.cap = static_cast<uint32_t>(s->wl_cap);
     ap.cont = s->cont;
     ap.st = s->st;
     ap.blim = s->blim;
@@ -593,7 +594,7 @@ bool server_step(irgl_server* s) {
     bp.qlast = s->qlast;
     bp.items[0] = s->items[0];
     bp.items[1] = s->items[1];
-    bp.cap = static_cast<uint32_t>(s->arena_n);
+    bp.cap = static_cast<uint32_t>(s->wl_cap);
     bp.cont = s->cont;
     bp.st = s->st;
     bp.tn = Tune{s->t.warp_thresh, s->t.cta_thresh, s->t.chunk, thread_bin(s->t)};
@@ -818,8 +819,10 @@ irgl_status irgl_server_create(irgl_ctx* ctx, const irgl_server_config* cfg, irg
     if (packed) e = cudaMalloc(&s->ds, sizeof(unsigned long long) * s->arena_n);
     else e = cudaMalloc(&s->stamp, sizeof(uint32_t) * s->arena_n);
   }
-  if (e == cudaSuccess) e = cudaMalloc(&s->items[0], sizeof(uint32_t) * s->arena_n);
-  if (e == cudaSuccess) e = cudaMalloc(&s->items[1], sizeof(uint32_t) * s->arena_n);
+  // with sub-rounds also room for what every CTA leaves of its last one (as in a batch)
+  s->wl_cap = std::min<uint64_t>(s->arena_n + (s->sub_rounds ? 2048ull * static_cast<uint64_t>(ctx->sm_count) : 0ull), 0xFFFFFFF0ull);
+  if (e == cudaSuccess) e = cudaMalloc(&s->items[0], sizeof(uint32_t) * s->wl_cap);
+  if (e == cudaSuccess) e = cudaMalloc(&s->items[1], sizeof(uint32_t) * s->wl_cap);
   if (e == cudaSuccess) e = cudaMalloc(&s->qlast, sizeof(uint32_t) * S);
   if (e == cudaSuccess) e = cudaMalloc(&s->cont, 128);
   if (nf && e == cudaSuccess) e = cudaMalloc(&s->far_items[0], sizeof(uint32_t) * s->arena_n);
